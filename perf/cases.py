@@ -118,41 +118,54 @@ def _hard_counts(case):
     return [1 + (case["hard"] - 1) * (b + 1) // B for b in range(B)]
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """Weights and inputs of a case; everything is drawn here, in this order."""
     g = GEOMETRIES[case["model"]]
     gen = torch.Generator(device="cuda")
     gen.manual_seed(int(seed))
     B, P, G, Lb = case["batch"], case["prompt"], case["gen"], case["block"]
     L, kind = P + G, case["kind"]
     sigma = 0.02 * math.sqrt(g.d_model)
-    model = jot.Model(g, _weights(g, 0 if kind == "head" else g.n_layers, gen), B, L)
-    s = {"case": case, "model": model, "bump_id": _token_ids(g, (B, L), gen)}
+    s = {"weights": _weights(g, 0 if kind == "head" else g.n_layers, gen), "bump_id": _token_ids(g, (B, L), gen)}
     uniform = torch.rand(B, L, device="cuda", generator=gen)
     if kind.startswith("generate"):
         order = torch.argsort(uniform[:, P:].reshape(B, G // Lb, Lb), dim=2)
         n_hard = torch.tensor(_hard_counts(case), device="cuda").view(B, 1, 1)
         val = torch.full((B, L), 30.0, device="cuda")
         val[:, P:] = torch.where(order < n_hard, 8.6 * sigma, 30.0).reshape(B, G)
-        s.update(bump_val=val, prompt=_token_ids(g, (B, P), gen), params=jot.Params(GENERATE_TAU, GENERATE_TAU, 0.5, 8))
-        if kind == "generate_cached":
-            model.attach_kv_cache()
+        s.update(bump_val=val, prompt=_token_ids(g, (B, P), gen))
         return s
     s["bump_val"] = 6.25 * sigma + 12.0 * uniform
-    s["params"] = jot.Params(*THRESHOLDS[case["model"]])
     lo, hi = _first_undecided_block(case)
     canvas = _token_ids(g, (B, L), gen)
     canvas[:, lo:] = g.mask_id                           # blocks before the current one are decided, later ones are not
     if kind == "head" and Lb > 32:                       # ... and so are some positions inside a long block
         decided = torch.rand(B, Lb, device="cuda", generator=gen) < 0.5
         canvas[:, lo:hi] = torch.where(decided, _token_ids(g, (B, Lb), gen), canvas[:, lo:hi])
-    s.update(canvas=canvas, tokens=canvas.clone(), stats=jot.Stats.empty(B, L, "cuda"), lo=lo, hi=hi,
-             n_masked=torch.zeros(B, dtype=torch.int32, device="cuda"))
+    s["canvas"] = canvas
     if kind == "head":
         s["hidden"] = torch.empty(B * L, g.d_model, dtype=torch.bfloat16, device="cuda").normal_(0.0, 1.0, generator=gen)
+    return s
+
+
+def prepare(case, seed):
+    s = _inputs(case, seed)
+    B, L, kind = case["batch"], case["prompt"] + case["gen"], case["kind"]
+    model = jot.Model(GEOMETRIES[case["model"]], s.pop("weights"), B, L)
+    s.update(case=case, model=model)
+    if kind.startswith("generate"):
+        s["params"] = jot.Params(GENERATE_TAU, GENERATE_TAU, 0.5, 8)
+        if kind == "generate_cached":
+            model.attach_kv_cache()
+        return s
+    lo, hi = _first_undecided_block(case)
+    s.update(params=jot.Params(*THRESHOLDS[case["model"]]), tokens=s["canvas"].clone(), stats=jot.Stats.empty(B, L, "cuda"),
+             lo=lo, hi=hi, n_masked=torch.zeros(B, dtype=torch.int32, device="cuda"))
+    if kind == "head":
         s["sampling"] = jot.Sampling(case["temperature"], int(seed), 3) if case["temperature"] > 0 else None
     if kind == "cached":
         model.attach_kv_cache()
-        model.denoise_step_cached(canvas, lo, hi, True)
+        model.denoise_step_cached(s["canvas"], lo, hi, True)
     return s
 
 
@@ -177,6 +190,69 @@ def run(s):
     out = {"tokens": tokens, "top1": stats.top1, "top2": stats.top2, "argmax": stats.argmax, "p1": 1.0 / stats.sumexp}
     if stats.sampled is not None:
         out["sampled"] = stats.sampled
+    return out
+
+
+# ------------------------------------------------------------------------------------------------ the same in 64 bits
+def _norm64(h, gain, eps):
+    return h * torch.rsqrt((h * h).mean(-1, keepdim=True) + eps) * gain.double()
+
+
+def _hidden64(g, w, canvas):
+    """The network on the whole canvas, with no activation rounded; final-normalised, [B * L, d]."""
+    B, L = canvas.shape
+    nq, nkv, hd = g.n_q_heads, g.n_kv_heads, g.head_dim
+    h = w["embed"][canvas.long()].double().reshape(B * L, -1)
+    inv = g.rope_theta ** (-torch.arange(hd // 2, dtype=torch.float64, device="cuda") * 2.0 / hd)
+    angle = torch.arange(L, dtype=torch.float64, device="cuda")[:, None, None] * inv
+    cos, sin = torch.cos(angle), torch.sin(angle)
+
+    def turn(t):
+        a, b = t[..., :hd // 2], t[..., hd // 2:]
+        return torch.cat([a * cos - b * sin, b * cos + a * sin], dim=-1)
+
+    for lw in w["layers"]:
+        qkv = (_norm64(h, lw["attn_norm"], g.rms_eps) @ lw["wqkv"].double().T).reshape(B, L, nq + 2 * nkv, hd)
+        o = torch.empty(B, L, nq * hd, dtype=torch.float64, device="cuda")
+        for b in range(B):
+            q, k, v = turn(qkv[b, :, :nq]), turn(qkv[b, :, nq:nq + nkv]), qkv[b, :, nq + nkv:]
+            q = q.reshape(L, nkv, nq // nkv, hd).permute(1, 2, 0, 3)                       # [kv head, its queries, L, hd]
+            scores = q @ k.permute(1, 2, 0)[:, None] / math.sqrt(hd)
+            o[b] = (torch.softmax(scores, -1) @ v.permute(1, 0, 2)[:, None]).permute(2, 0, 1, 3).reshape(L, nq * hd)
+        h = h + o.reshape(B * L, -1) @ lw["wo"].double().T
+        gate_up = _norm64(h, lw["mlp_norm"], g.rms_eps) @ lw["w_gate_up"].double().T
+        act = torch.nn.functional.silu(gate_up[:, :g.d_ff]).mul_(gate_up[:, g.d_ff:])
+        h = h + act @ lw["w_down"].double().T
+        del gate_up, act
+    return _norm64(h, w["final_norm"], g.rms_eps)
+
+
+def exact(case, seed):
+    """Statistics of the masked positions of the block as 64 bits give them.  Tokens and argmax have no such value
+    (a tie or a threshold decides them); a block pass right after the full pass sees what the full pass saw."""
+    if case["kind"].startswith("generate"):
+        return None
+    g, s = GEOMETRIES[case["model"]], _inputs(case, seed)
+    lo, hi = _first_undecided_block(case)
+    canvas, w = s["canvas"], s["weights"]
+    masked = torch.zeros_like(canvas, dtype=torch.bool)
+    masked[:, lo:hi] = canvas[:, lo:hi] == g.mask_id
+    rows = masked.flatten().nonzero().flatten()
+    hidden = s["hidden"].double() if case["kind"] == "head" else _hidden64(g, w, canvas)
+    hidden, head = hidden[rows], w["lm_head"].double()
+    out = {"top1": torch.zeros(canvas.shape, dtype=torch.float64, device="cuda"), "p1": torch.ones(canvas.shape, dtype=torch.float64, device="cuda")}
+    out["top2"] = out["top1"].clone()
+    for at in range(0, len(rows), 256):
+        r = rows[at:at + 256]
+        logits = hidden[at:at + 256] @ head.T
+        logits[torch.arange(len(r), device="cuda"), s["bump_id"].flatten()[r].long()] += s["bump_val"].flatten()[r].double()
+        logits[:, g.mask_id] = -math.inf
+        best = logits.topk(2, dim=1).values
+        out["top1"].view(-1)[r], out["top2"].view(-1)[r] = best[:, 0], best[:, 1]
+        out["p1"].view(-1)[r] = torch.exp(best[:, 0] - torch.logsumexp(logits, 1))
+    out.update(tokens=None, argmax=None)
+    if case["temperature"] > 0:
+        out["sampled"] = None
     return out
 
 
