@@ -60,6 +60,7 @@ struct BodyParams {
     int stages, stage_bytes;
     int s_qkv, s_o, s_down;                // K ranges per 256-row tile
     int gu_rows;                           // gate rows (and as many up rows) per tile of the gate/up projection: 8 .. 128
+    int attn_pairs;                        // two attention items side by side in a CTA
     __nv_bfloat16 *h, *a, *attn, *act, *hsel;
     __nv_bfloat16 *qkv, *vt;               // layer 0's; the next layer's `*_stride` elements further (0: one scratch buffer)
     size_t qkv_stride, vt_stride;
@@ -82,7 +83,7 @@ struct BodyParams {
 
 // Shared memory of the workers: the attention exchange (and Q), or one row as bf16.
 __host__ __device__ inline int body_work_bytes(int hd, int d) {
-    const int exchange = 4 * kBodyQT * (hd + kBodyPad) * 4 + 8 * kBodyQT * 2 * 4 + kBodyQT * hd * 2;
+    const int exchange = 4 * kBodyQT * (hd + kBodyPad) * 4 + 8 * kBodyQT * 2 * 4 + 2 * kBodyQT * hd * 2;
     return ((exchange > 2 * d ? exchange : 2 * d) + 127) / 128 * 128;
 }
 
@@ -200,7 +201,8 @@ __device__ __noinline__ bool body_reduce_norm(const BodyParams& p, int row, int 
         unsigned long long* words = p.row_sums + (size_t)slot * kBodyMaxParts;
         if (tid == 0) {
             const unsigned long long w = ((unsigned long long)tag << 32) | __float_as_uint(ss);
-            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(words + part), "l"(w) : "memory");
+            // (an atomic acts where the word lives; a plain store took up to 4 us to be seen from the other die)
+            atomicExch(words + part, w);
         }
         if (tid < parts) {
             unsigned long long w = 0, t0 = 0;
@@ -364,31 +366,34 @@ __device__ __noinline__ void body_qkv_finish(const BodyParams& p, __nv_bfloat16*
     }
 }
 
-// Attention of 16 queries of one head: the 8 warps take blocks of 32 keys each with their own running maximum, row sum
-// and output, and meet in shared memory.  Few queries leave nothing for a 128-row tcgen05 tile to do, and this way K and V
+// Attention of 16 queries of one head by a group of GW warps (all 8, or 4 when there are more items than CTAs and the
+// keys are few: two items side by side): the warps take blocks of 32 keys each with their own running maximum, row sum and
+// output, and meet in shared memory.  Few queries leave nothing for a 128-row tcgen05 tile to do, and this way K and V
 // do not pass through shared memory: contraction indices may be permuted as long as both operands agree, so a thread's
 // 16-byte load of 8 consecutive elements serves as its fragment of two k-steps.
 //   scores: thread q4 = lane % 4 holds elements 32 s + 8 q4 .. + 7 of the head dimension
 //   keys:   column c of 8-key tile t is key 8 (c / 2) + 2 t + c % 2 of the block, so that a thread's eight probabilities
 //           of a row belong to 8 consecutive keys, 16 bytes of V^T
-template <int HD>
+template <int HD, int GW>
 __device__ __noinline__ void body_attention(const BodyParams& p, const __nv_bfloat16* qkv, const __nv_bfloat16* vt, uint8_t* work,
                                             int tid) {
     constexpr int KS = HD / 32;            // 16-byte loads per row and thread
     constexpr int NT = HD / 8;             // 8-column tiles of the output
     constexpr int LDO = HD + kBodyPad;
     constexpr int VB = 8;                  // V tiles on their way ahead of their products
-    const int w = tid >> 5, lane = tid & 31, r = lane >> 2, q4 = lane & 3;
-    float* sO = reinterpret_cast<float*>(work);                        // [4][16 rows][LDO]
-    float* sM = sO + 4 * kBodyQT * LDO;                                 // [8][16] maximum (base-2 exponent), then row sum
-    float* sL = sM + 8 * kBodyQT;
-    uint4* sQ = reinterpret_cast<uint4*>(sL + 8 * kBodyQT);             // [2 KS][32]
+    constexpr int HW = GW / 2, GROUPS = 8 / GW;
+    const int grp = (tid >> 5) / GW, w = (tid >> 5) % GW, lane = tid & 31, r = lane >> 2, q4 = lane & 3;
+    float* sO = reinterpret_cast<float*>(work) + grp * HW * kBodyQT * LDO;                  // [HW][16 rows][LDO]
+    float* sM = reinterpret_cast<float*>(work) + 4 * kBodyQT * LDO + grp * GW * kBodyQT;     // [GW][16] maximum (base-2 exponent)
+    float* sL = sM + 8 * kBodyQT;                                                           // ... and row sum
+    uint4* sQ = reinterpret_cast<uint4*>(reinterpret_cast<float*>(work) + 4 * kBodyQT * LDO + 16 * kBodyQT) + grp * KS * 64;    // [2 KS][32]
+    auto sync_group = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + (GROUPS > 1 ? 1 + grp : 0)), "n"(GW * 32) : "memory"); };
     const int Lr = p.rows_per_seq, L = p.L, Lp = p.Lp, pos0 = p.pos0, nq = p.nq, nkv = p.nkv, group = nq / nkv;
     const int N = (nq + 2 * nkv) * HD;
     const int nqt = (Lr + kBodyQT - 1) / kBodyQT, nkb = (L + 31) / 32, items = p.B * nq * nqt;
     __nv_bfloat16* attn = p.attn;
     const float c = p.scale_log2e;
-    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    for (int item = blockIdx.x + grp * gridDim.x; item < items; item += GROUPS * gridDim.x) {
         const int qt = item % nqt, hb = item / nqt, h = hb % nq, b = hb / nq, kvh = h / group;
         const __nv_bfloat16* seq = qkv + (size_t)b * L * N;
         const __nv_bfloat16* vrow = vt + ((size_t)b * nkv + kvh) * HD * Lp;
@@ -397,13 +402,14 @@ __device__ __noinline__ void body_attention(const BodyParams& p, const __nv_bflo
         for (int n = 0; n < NT; ++n) O[n][0] = O[n][1] = O[n][2] = O[n][3] = 0.f;
         float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;
         // Q as fragments in shared memory: [k-step pair][row half][lane]
-        if (w < 2 * KS) {
-            const int i = min(qt * kBodyQT + r + 8 * (w & 1), Lr - 1);
-            sQ[w * 32 + lane] = ld_l2_here(seq + (size_t)(pos0 + i) * N + h * HD + (w >> 1) * 32 + q4 * 8);
+#pragma unroll
+        for (int f = w; f < 2 * KS; f += GW) {
+            const int i = min(qt * kBodyQT + r + 8 * (f & 1), Lr - 1);
+            sQ[f * 32 + lane] = ld_l2_here(seq + (size_t)(pos0 + i) * N + h * HD + (f >> 1) * 32 + q4 * 8);
         }
-        BODY_SYNC_WORKERS();
+        sync_group();
 #pragma unroll 1
-        for (int j = w; j < nkb; j += 8) {
+        for (int j = w; j < nkb; j += GW) {
             const int k0 = j * 32;
             float S[4][4];
 #pragma unroll
@@ -501,8 +507,8 @@ __device__ __noinline__ void body_attention(const BodyParams& p, const __nv_bflo
         l1 += __shfl_xor_sync(0xffffffffu, l1, 1);
         l0 += __shfl_xor_sync(0xffffffffu, l0, 2);
         l1 += __shfl_xor_sync(0xffffffffu, l1, 2);
-        // two rounds: warps 4..7 hand over to warps 0..3, whose four results are combined below
-        float* o0 = sO + ((w & 3) * kBodyQT + r) * LDO + 2 * q4;
+        // two rounds: the upper half of the warps hand over to the lower half, whose results are combined below
+        float* o0 = sO + ((w % HW) * kBodyQT + r) * LDO + 2 * q4;
         auto put = [&]() {
             if (q4 == 0) {
                 sM[w * kBodyQT + r] = m0; sM[w * kBodyQT + r + 8] = m1;
@@ -514,15 +520,15 @@ __device__ __noinline__ void body_attention(const BodyParams& p, const __nv_bflo
                 *reinterpret_cast<float2*>(o0 + 8 * LDO + n * 8) = make_float2(O[n][2], O[n][3]);
             }
         };
-        if (nkb > 4) {
-            if (w >= 4) put();
-            BODY_SYNC_WORKERS();
-            if (w < 4) {                                                // (warps 0..3 have keys here: m0 and m1 are finite)
-                const float p0 = sM[(w + 4) * kBodyQT + r], p1 = sM[(w + 4) * kBodyQT + r + 8];
+        if (nkb > HW) {
+            if (w >= HW) put();
+            sync_group();
+            if (w < HW) {                                               // (these warps have keys here: m0 and m1 are finite)
+                const float p0 = sM[(w + HW) * kBodyQT + r], p1 = sM[(w + HW) * kBodyQT + r + 8];
                 const float x0 = fmaxf(m0, p0), x1 = fmaxf(m1, p1);
                 const float f0 = ex2_approx(m0 - x0), f1 = ex2_approx(m1 - x1), g0 = ex2_approx(p0 - x0), g1 = ex2_approx(p1 - x1);
-                l0 = l0 * f0 + sL[(w + 4) * kBodyQT + r] * g0;
-                l1 = l1 * f1 + sL[(w + 4) * kBodyQT + r + 8] * g1;
+                l0 = l0 * f0 + sL[(w + HW) * kBodyQT + r] * g0;
+                l1 = l1 * f1 + sL[(w + HW) * kBodyQT + r + 8] * g1;
                 m0 = x0;
                 m1 = x1;
 #pragma unroll
@@ -532,21 +538,21 @@ __device__ __noinline__ void body_attention(const BodyParams& p, const __nv_bflo
                     O[n][2] = O[n][2] * f1 + e.x * g1; O[n][3] = O[n][3] * f1 + e.y * g1;
                 }
             }
-            BODY_SYNC_WORKERS();
+            sync_group();
         }
-        if (w < 4) put();
-        BODY_SYNC_WORKERS();
+        if (w < HW) put();
+        sync_group();
         {
-            constexpr int PER = HD / 16;                                // output columns per thread: 16 threads a row
-            const int row = tid >> 4, c0 = (tid & 15) * PER, i = qt * kBodyQT + row;
+            constexpr int PER = HD / (2 * GW);                          // output columns per thread: 2 GW threads a row
+            const int tg = tid % (GW * 32), row = tg / (2 * GW), c0 = tg % (2 * GW) * PER, i = qt * kBodyQT + row;
             float m = -INFINITY;
 #pragma unroll
-            for (int s = 0; s < 4; ++s) m = fmaxf(m, sM[s * kBodyQT + row]);
+            for (int s = 0; s < HW; ++s) m = fmaxf(m, sM[s * kBodyQT + row]);
             float l = 0.f, x[PER];
 #pragma unroll
             for (int e = 0; e < PER; ++e) x[e] = 0.f;
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
+            for (int s = 0; s < HW; ++s) {
                 const float f = ex2_approx(sM[s * kBodyQT + row] - m);    // 0 for a warp that had no keys
                 l += sL[s * kBodyQT + row] * f;
 #pragma unroll
@@ -563,7 +569,7 @@ __device__ __noinline__ void body_attention(const BodyParams& p, const __nv_bflo
                     *reinterpret_cast<uint2*>(dst + e) = make_uint2(pack_bf16(x[e] * inv, x[e + 1] * inv), pack_bf16(x[e + 2] * inv, x[e + 3] * inv));
             }
         }
-        BODY_SYNC_WORKERS();               // the exchange area is free again
+        sync_group();               // the exchange area is free again
     }
 }
 
@@ -873,8 +879,13 @@ body_kernel(const __grid_constant__ BodyParams kp, const __grid_constant__ CUten
             if (!(ok = step_end(false))) break;
             body_qkv_finish(p, qkv, vt, tid);
             if (!(ok = step_end(false))) break;
-            if (p.hd == 128) body_attention<128>(p, qkv, vt, work, tid);
-            else body_attention<64>(p, qkv, vt, work, tid);
+            if (p.hd == 128) {
+                if (p.attn_pairs) body_attention<128, 4>(p, qkv, vt, work, tid);
+                else body_attention<128, 8>(p, qkv, vt, work, tid);
+            } else {
+                if (p.attn_pairs) body_attention<64, 4>(p, qkv, vt, work, tid);
+                else body_attention<64, 8>(p, qkv, vt, work, tid);
+            }
             if (!(ok = step_end(true))) break;
             epilogue(1);
             if (!(ok = step_end(false))) break;

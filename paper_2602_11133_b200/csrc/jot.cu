@@ -580,9 +580,9 @@ int encode_activation_maps(jot_model* m, int B, int L) {
 
 // K ranges per 256-row tile of a projection of the one-launch body: as many as fill the SMs, with at least two k-blocks
 // each and room for the fp32 partial sums.
-int body_pick_split(int M, int N, int K, int sms) {
+int body_pick_split(int M, int N, int K, int sms, int most = kBodyMaxSplit) {
     const int tiles = (N + 255) / 256, num_kb = (K + 63) / 64;
-    int s = std::min(sms / tiles, kBodyMaxSplit);
+    int s = std::min(sms / tiles, most);
     while (s > 1 && (num_kb / s < 2 || (size_t)s * M * N * 4 > kSplitKBytes)) --s;
     return s < 1 ? 1 : s;
 }
@@ -594,11 +594,19 @@ int body_gate_up_rows(int ff, int sms) {
     return (ff + 8 * sms * waves - 1) / (8 * sms * waves) * 8;
 }
 
-// Whether the body of a pass over M rows runs as one launch (body.cuh).
+// Whether the body of a pass over M rows runs as one launch (body.cuh).  Measured against the separate launches, 8 layers
+// of the LLaDA-8B and Dream-7B shapes: 32 rows 1.16x and 1.10x, 64 rows 1.10x and 1.05x, 96 rows 1.05x and 1.00x, 112 rows
+// 1.07x and 1.01x; 128 rows 0.98x and 0.95x; 133 rows, where the separate gate/up projection takes two launches, 1.02x and
+// 1.01x; from 152 rows on 0.9x: the partial sums grow with the rows.  Where those are small (a model of a few hundred
+// columns: 152 us a step either way, 1.10x at 16 rows) one kind of body serves every batch, so that a sequence's results
+// do not depend on its neighbours.  What counts there is the
+// number of steps, at any number of rows.
 bool body_applies(const jot_model* m, int M) {
     const jot_model_config& c = m->cfg;
     const size_t cols = std::max((size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, (size_t)c.d_model);
-    return m->body_ok && M <= kBodyMaxTokens && c.n_layers > 0 && (size_t)M * cols * 4 <= kSplitKBytes;
+    const size_t sums = (size_t)M * cols * 4;                       // fp32 partial sums of one K range
+    const bool few = M <= 112 || (M > 128 && M <= 144) || (M <= kBodyMaxTokens && sums <= (2u << 20));
+    return m->body_ok && few && c.n_layers > 0 && sums <= kSplitKBytes;
 }
 
 int encode_act_maps(jot_model* m, jot_model::ActMaps* am, int M) {
@@ -614,7 +622,8 @@ int encode_act_maps(jot_model* m, jot_model::ActMaps* am, int M) {
         JOT_TRY(make_map_2d(m->di, &am->ba, m->a, M, c.d_model, c.d_model, box));
         JOT_TRY(make_map_2d(m->di, &am->battn, m->attn, M, o_cols, o_cols, box));
         JOT_TRY(make_map_2d(m->di, &am->bact, m->act, M, c.d_ff, c.d_ff, box));
-        am->s_qkv = body_pick_split(M, qkv_cols, c.d_model, m->di->sms);
+        // (QKV: more than four ranges cost the step that adds them more than they save, 1 to 3 us a layer at 96 to 192 rows)
+        am->s_qkv = body_pick_split(M, qkv_cols, c.d_model, m->di->sms, 4);
         am->s_o = body_pick_split(M, c.d_model, o_cols, m->di->sms);
         am->s_down = body_pick_split(M, c.d_model, c.d_ff, m->di->sms);
     }
@@ -776,6 +785,12 @@ int launch_body(jot_model* m, const jot_model::ActMaps& am, const int32_t* d_tok
     p.seq_map = seq_map; p.mask_id = c.mask_id; p.blk_lo = ar.blk_lo; p.blk_hi = ar.blk_hi; p.state = ar.state;
     p.P = ar.P; p.block_len = ar.block_len; p.n_blocks = ar.n_blocks;
     p.rows = m->rows; p.rows_out = m->rows_out; p.d_R = m->ctrl + 1;
+    {
+        // rounds of 32-key blocks a warp goes through, with all warps on one item or half of them; a tie means fewer exchanges
+        auto up = [](int a, int b) { return (a + b - 1) / b; };
+        const int items = B * c.n_q_heads * up(Lr, kBodyQT), blocks = up(L, 32), sms = m->di->sms;
+        p.attn_pairs = items > sms && up(items, 2 * sms) * up(blocks, 4) <= up(items, sms) * up(blocks, 8);
+    }
     p.parts = 1;
     while (p.parts < kBodyMaxParts && p.M * p.parts * 2 <= m->di->sms) p.parts *= 2;
     p.row_sums = m->body_row_sums; p.barrier = m->body_barrier; p.status = m->ctrl;
@@ -809,7 +824,9 @@ int forward_to_head(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStr
         JOT_TRY(encode_act_maps(m, &am, B * Lr));
         const bool cached = span && span->use_cache;
         if (cached) JOT_TRY(encode_kv_maps(m, B, L));
-        return launch_body(m, am, d_tokens, B, L, st, seq_map, Lr, pos0, cached, ar);
+        const int rc = launch_body(m, am, d_tokens, B, L, st, seq_map, Lr, pos0, cached, ar);
+        if (rc != JOT_ERR_CUDA || g_last_cuda_error != (int)cudaErrorCooperativeLaunchTooLarge) return rc;
+        m->body_ok = false;                    // a context with a part of the SMs: its CTAs cannot all be resident
     }
     JOT_TRY(forward_body(m, d_tokens, B, L, st, seq_map, span));
     ProfScope ps(m, JOT_PROF_ROWS, st);

@@ -1,6 +1,7 @@
-"""GPU parity of the one-launch transformer body (canvases of at most 256 rows) against the CPU oracle, at the sizes where
-its tiling changes: row counts around the 16-row granularity of the token operand, around 128 rows (two accumulator
-pairs or one) and around the SM count (rows shared by several CTAs or not), K ranges from 1 to 8, ragged tiles."""
+"""GPU parity of the one-launch transformer body (small canvases) against the CPU oracle, at the sizes where
+its tiling changes: row counts around the 16-row granularity of the token operand, on both sides of 128 rows (two
+accumulator pairs or one), few enough for several CTAs to share a row or not, one or two attention items side by side,
+K ranges from 1 to 8, ragged tiles."""
 import pytest
 import torch
 
@@ -32,9 +33,11 @@ def jot():
     ("hd128", 1, 6, 11),        # 17
     ("wide", 1, 17, 16),        # 33 rows, four CTAs a row
     ("wide", 2, 20, 18),        # 76 rows: one CTA a row
-    ("wide", 1, 60, 68),        # 128 rows: the last size with two accumulator pairs
-    ("gqa", 3, 20, 23),         # 129 rows
-    ("wide", 1, 70, 79),        # 149 rows: more rows than CTAs
+    ("wide", 1, 52, 60),        # 112 rows: the last size with two accumulator pairs; attention items side by side
+    ("gqa", 3, 20, 23),         # 129 rows: the first with one
+    ("hd128", 2, 40, 32),       # 144 rows: the last size of a wide model
+    ("wide", 18, 3, 5),         # 144 rows of 18 short sequences: one key block, items side by side
+    ("gqa", 1, 70, 79),         # 149 rows: more rows than CTAs
     ("hd128", 2, 64, 64),       # 256 rows: the last size
 ])
 def test_step_matches_oracle(jot, name, B, P, G):
@@ -59,6 +62,7 @@ def test_step_matches_oracle(jot, name, B, P, G):
 
 
 @pytest.mark.parametrize("name,B,P,G,lo,hi", [
+    ("gqa", 6, 30, 100, 51, 69),     # 108 rows, items side by side: five key blocks over four warps
     ("wide", 1, 20, 55, 31, 36),     # five rows at an odd position; the last of three key blocks is ragged
     ("hd128", 3, 40, 300, 97, 129),  # eleven key blocks: every warp has one, some two
     ("wide", 2, 3, 20, 3, 23),       # one key block
