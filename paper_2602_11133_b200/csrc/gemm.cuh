@@ -272,10 +272,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t t_ac
                         __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&ov);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            float g0 = g[q * 8 + 2 * j], g1 = g[q * 8 + 2 * j + 1];
-                            float a0 = g0 / (1.f + __expf(-g0)) * u[q * 8 + 2 * j];
-                            float a1 = g1 / (1.f + __expf(-g1)) * u[q * 8 + 2 * j + 1];
-                            o2[j] = __floats2bfloat162_rn(a0, a1);
+                            const int e = q * 8 + 2 * j;
+                            o2[j] = __floats2bfloat162_rn(silu_mul(g[e], u[e]), silu_mul(g[e + 1], u[e + 1]));
                         }
                         *reinterpret_cast<uint4*>(dst + q * 8) = ov;
                     }

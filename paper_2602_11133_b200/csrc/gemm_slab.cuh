@@ -453,8 +453,8 @@ gemm_slab_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmW, co
                         __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&ov);
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            const float a0 = gg[2 * j] / (1.f + __expf(-gg[2 * j])) * uu[2 * j];
-                            const float a1 = gg[2 * j + 1] / (1.f + __expf(-gg[2 * j + 1])) * uu[2 * j + 1];
+                            const float a0 = silu_mul(gg[2 * j], uu[2 * j]);
+                            const float a1 = silu_mul(gg[2 * j + 1], uu[2 * j + 1]);
                             o2[j] = __floats2bfloat162_rn(a0, a1);
                         }
                         *reinterpret_cast<uint4*>(p.C + (size_t)t * p.ldc + oc) = ov;
@@ -733,8 +733,8 @@ gemm_slab_gateup2_kernel(const GemmParams p, const __grid_constant__ CUtensorMap
                     __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&ov);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float a0 = gg[2 * j] / (1.f + __expf(-gg[2 * j])) * uu[2 * j];
-                        const float a1 = gg[2 * j + 1] / (1.f + __expf(-gg[2 * j + 1])) * uu[2 * j + 1];
+                        const float a0 = silu_mul(gg[2 * j], uu[2 * j]);
+                        const float a1 = silu_mul(gg[2 * j + 1], uu[2 * j + 1]);
                         o2[j] = __floats2bfloat162_rn(a0, a1);
                     }
                     *reinterpret_cast<uint4*>(p.C + (size_t)t * p.ldc + oc) = ov;
