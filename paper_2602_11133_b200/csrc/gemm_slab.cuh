@@ -381,26 +381,28 @@ gemm_slab_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmW, co
                         staged = false;
                         const int kvh = head - p.nq - p.nkv, dd = (f0 + f_in) % p.hd;
                         if (f0 + f_in < p.N) {
-                            const int seq0 = t0 / p.rows_per_seq, pos_first = p.pos0 + (t0 - seq0 * p.rows_per_seq);
-                            const bool one_seq = (t0 + 31) / p.rows_per_seq == seq0 && t0 + 31 < p.M;
-                            __nv_bfloat16* row = p.vt + ((size_t)(seq0 * p.nkv + kvh) * p.hd + dd) * p.Lp + pos_first;
-                            if (one_seq && (pos_first & 7) == 0) {
+                            // (one division per chunk: one per token made a ragged last chunk cost 10 us)
+                            const int n_here = min(32, p.M - t0);
+                            int seq = t0 / p.rows_per_seq, at = t0 - seq * p.rows_per_seq;
+                            const size_t seq_step = (size_t)p.nkv * p.hd * p.Lp;
+                            __nv_bfloat16* row = p.vt + seq * seq_step + ((size_t)kvh * p.hd + dd) * p.Lp + p.pos0;
+                            const bool packed = at + n_here <= p.rows_per_seq && ((p.pos0 + at) & 7) == 0;
 #pragma unroll
-                                for (int q4 = 0; q4 < 4; ++q4) {
+                            for (int q4 = 0; q4 < 4; ++q4) {
+                                if (packed && q4 * 8 + 8 <= n_here) {
                                     uint4 ov;
                                     __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&ov);
 #pragma unroll
                                     for (int j = 0; j < 4; ++j) o2[j] = __floats2bfloat162_rn(v[q4 * 8 + 2 * j], v[q4 * 8 + 2 * j + 1]);
-                                    *reinterpret_cast<uint4*>(row + q4 * 8) = ov;
-                                }
-                            } else {
+                                    *reinterpret_cast<uint4*>(row + at) = ov;
+                                    at += 8;
+                                } else {
 #pragma unroll
-                                for (int j = 0; j < 32; ++j) {
-                                    const int t = t0 + j;
-                                    if (t < p.M) {
-                                        const int seq = t / p.rows_per_seq, pos = p.pos0 + (t - seq * p.rows_per_seq);
-                                        p.vt[((size_t)(seq * p.nkv + kvh) * p.hd + dd) * p.Lp + pos] = __float2bfloat16_rn(v[j]);
-                                    }
+                                    for (int j = 0; j < 8; ++j)
+                                        if (q4 * 8 + j < n_here) {
+                                            if (at == p.rows_per_seq) { at = 0; row += seq_step; }
+                                            row[at++] = __float2bfloat16_rn(v[q4 * 8 + j]);
+                                        }
                                 }
                             }
                         }
