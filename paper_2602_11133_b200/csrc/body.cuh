@@ -1,7 +1,7 @@
-// The whole transformer body of a small canvas (at most 256 rows) as ONE persistent kernel.
+// The whole transformer body of a small canvas (at most 64 rows) as ONE persistent kernel.
 //
 // With few rows a pass is a stream of the weights, and as separate launches every projection pays a launch, a pipeline
-// fill, a drain and an epilogue that nothing overlaps (7-10 us each at 32 rows, seven launches a layer).  Here one CTA per
+// fill, a drain and an epilogue that nothing overlaps (7-10 us each at 32 rows, seven launches a layer; 132 us a layer of the LLaDA-8B shape, 66 us for the bytes; here 107 us).  Here one CTA per
 // SM stays for the whole pass; the steps of a layer follow each other through a grid-wide barrier (1.3-1.8 us), and the
 // producer requests the first weight tiles of the next projection while the other roles are still in the steps before it
 // (weights are nobody's output; only the token tiles wait for the barrier).
@@ -32,7 +32,7 @@ namespace jot {
 
 constexpr int kBodyThreads = 384;
 constexpr int kBodyWorkers = 256;
-constexpr int kBodyMaxTokens = 256;        // two accumulators of 256 fp32 columns fill tensor memory
+constexpr int kBodyMaxTokens = 64;         // beyond that the separate launches are the faster ones (body_applies)
 constexpr int kBodyMaxStages = 8;
 constexpr int kBodyMaxSmem = 226 * 1024;   // dynamic part; the static barriers take the rest of the 227 KB
 constexpr int kBodyWTile = 256 * 128;      // bytes of W per stage: 256 rows x 64 bf16
@@ -605,7 +605,7 @@ body_kernel(const __grid_constant__ BodyParams kp, const __grid_constant__ CUten
         tma_prefetch_desc(&tmAct);
     }
     if (warp == 1) {
-        tmem_alloc(&tmem_base_slot, 512);
+        tmem_alloc(&tmem_base_slot, 256);
         tmem_relinquish();
     }
     tc_fence_before();
@@ -618,7 +618,8 @@ body_kernel(const __grid_constant__ BodyParams kp, const __grid_constant__ CUten
     const unsigned long long seen = grid_count(p.barrier), base = seen - seen % (unsigned long long)G;
     auto target = [&](int n_done) { return base + (unsigned long long)n_done * G; };       // n_done barriers complete
     const uint32_t acc_cols = (uint32_t)(p.n_tok + 31) & ~31u;                              // one accumulator of 128 weight rows
-    const int n_buf = p.n_tok <= 128 ? 2 : 1;                                               // accumulator pairs in tensor memory
+    constexpr int n_buf = 2, TMEM_COLS = 256;                                               // two pairs of accumulators
+    static_assert(2 * n_buf * kBodyMaxTokens <= TMEM_COLS, "accumulators fit");
 
     // ---- the four projections (0 QKV, 1 O, 2 gate/up, 3 down): tiles of weight rows, K ranges per tile, k-blocks ----
     const int qkv_cols = (p.nq + 2 * p.nkv) * p.hd, kd = (p.d + 63) / 64, ko = (p.nq * p.hd + 63) / 64, kf = (p.ff + 63) / 64;
@@ -911,7 +912,7 @@ body_kernel(const __grid_constant__ BodyParams kp, const __grid_constant__ CUten
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
+        tmem_dealloc(tmem_base, TMEM_COLS);
     }
     if (threadIdx.x == 0 && abort_flag) atomicExch(p.status, kBodyStatus);
 }

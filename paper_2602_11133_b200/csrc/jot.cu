@@ -594,19 +594,18 @@ int body_gate_up_rows(int ff, int sms) {
     return (ff + 8 * sms * waves - 1) / (8 * sms * waves) * 8;
 }
 
-// Whether the body of a pass over M rows runs as one launch (body.cuh).  Measured against the separate launches, 8 layers
-// of the LLaDA-8B and Dream-7B shapes: 32 rows 1.16x and 1.10x, 64 rows 1.10x and 1.05x, 96 rows 1.05x and 1.00x, 112 rows
-// 1.07x and 1.01x; 128 rows 0.98x and 0.95x; 133 rows, where the separate gate/up projection takes two launches, 1.02x and
-// 1.01x; from 152 rows on 0.9x: the partial sums grow with the rows.  Where those are small (a model of a few hundred
-// columns: 152 us a step either way, 1.10x at 16 rows) one kind of body serves every batch, so that a sequence's results
-// do not depend on its neighbours.  What counts there is the
-// number of steps, at any number of rows.
+// Whether the body of a pass over M rows runs as one launch (body.cuh): few rows, and layers whose weights take HBM longer
+// than the barriers cost.  One launch against separate ones, us for 8 layers and a head: LLaDA-8B shape (436 MB a layer)
+// 1078 / 1193 at 32 rows, 1130 / 1204 at 64, 1223 / 1241 at 96, 1300 / 1270 at 128; Dream-7B shape (466 MB) 1096 / 1160 at 32,
+// 1155 / 1162 at 64, 1200 / 1184 at 80; 2048 columns (103 MB) 561 / 593 at 32, 638 / 612 at 80; 1024 columns (26 MB) 454 / 462
+// at 32, 493 / 478 at 80; 512 columns (6 MB) 394 / 371.  More rows mean more partial sums and more of the step between the
+// projections; small layers have nothing to stream meanwhile.
 bool body_applies(const jot_model* m, int M) {
     const jot_model_config& c = m->cfg;
-    const size_t cols = std::max((size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, (size_t)c.d_model);
-    const size_t sums = (size_t)M * cols * 4;                       // fp32 partial sums of one K range
-    const bool few = M <= 112 || (M > 128 && M <= 144) || (M <= kBodyMaxTokens && sums <= (2u << 20));
-    return m->body_ok && few && c.n_layers > 0 && sums <= kSplitKBytes;
+    const size_t qkv = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, o = (size_t)c.n_q_heads * c.head_dim;
+    const size_t layer_bytes = 2 * ((qkv + o) * c.d_model + 3 * (size_t)c.d_ff * c.d_model);
+    return m->body_ok && c.n_layers > 0 && M <= kBodyMaxTokens && layer_bytes >= ((size_t)96 << 20) &&
+           M * std::max(qkv, (size_t)c.d_model) * 4 <= kSplitKBytes;
 }
 
 int encode_act_maps(jot_model* m, jot_model::ActMaps* am, int M) {
@@ -622,7 +621,7 @@ int encode_act_maps(jot_model* m, jot_model::ActMaps* am, int M) {
         JOT_TRY(make_map_2d(m->di, &am->ba, m->a, M, c.d_model, c.d_model, box));
         JOT_TRY(make_map_2d(m->di, &am->battn, m->attn, M, o_cols, o_cols, box));
         JOT_TRY(make_map_2d(m->di, &am->bact, m->act, M, c.d_ff, c.d_ff, box));
-        // (QKV: more than four ranges cost the step that adds them more than they save, 1 to 3 us a layer at 96 to 192 rows)
+        // (QKV: more than four ranges cost the step that adds them as much as they save)
         am->s_qkv = body_pick_split(M, qkv_cols, c.d_model, m->di->sms, 4);
         am->s_o = body_pick_split(M, c.d_model, o_cols, m->di->sms);
         am->s_down = body_pick_split(M, c.d_model, c.d_ff, m->di->sms);
