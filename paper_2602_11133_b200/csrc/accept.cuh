@@ -81,8 +81,8 @@ __device__ __forceinline__ AcceptParamsDev accept_pick_params(const AcceptArgs& 
 
 // The kernel is a chain of memory round trips and barriers over a few hundred numbers, so it is kept short: everything a
 // decision reads is requested before the canvas has arrived, thread t looks after position lo + t of the block (no list of
-// candidates is built), and the ranks are counted by all threads together.  6.6 -> 4.9 us for a block of 64, 8.7 before as
-// ncu times it cold.
+// candidates is built), and the ranks are counted by all threads together: 8.3 -> 5.8 us for a block of 32 in a canvas of 384
+// as ncu times it.
 // Dynamic shared memory: resolved bitmap words; per position of the block its rank, sum-exp (not a number where there is
 // nothing to rank: no comparison with it holds) and flags.
 template <bool INLINE>
@@ -241,7 +241,7 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
         const int n4 = (n_pos + 3) >> 2, o_lo = n4 * q / share, o_hi = n4 * (q + 1) / share;
         for (int c = tid % W; c < n_pos; c += W) {
             const float Sc = pos_S[c];
-            if (!(Sc == Sc)) continue;
+            if (!(Sc == Sc)) continue;                         // nothing to rank here; a sum that is no number ranks first
             int before = 0;
             for (int o = o_lo; o < o_hi; ++o) {
                 const float4 v = reinterpret_cast<const float4*>(pos_S)[o];
@@ -259,8 +259,9 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
     // freeze: chosen candidates receive their argmax; everything else is left untouched
     int my_final = 0;
     for (int c = tid; c < n_pos; c += blockDim.x) {
-        const float S = pos_S[c];
-        const uint8_t f = flag[c] | ((k_eff > 0 && S == S && rank[c] < k_eff) ? 2 : 0);
+        const uint8_t exited = flag[c];
+        const bool ranked = k_eff > 0 && is_cand(c) && !(prm.schedule_after_exit && (exited & 1));
+        const uint8_t f = exited | ((ranked && rank[c] < k_eff) ? 2 : 0);
         if (f) {
             const int i = lo + c;
             const size_t gi = row + i;
@@ -296,6 +297,10 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
     }
 }
 
+// The longest canvas taken: 9 bytes a position and a bit in 200 KB.
+inline bool accept_length_ok(int L) {
+    return (size_t)((L + 31) / 32 + 2) * 4 + (size_t)L * 8 + (size_t)((L + 3) / 4) * 4 + 16 <= 200 * 1024;
+}
 inline size_t accept_smem_bytes(int L) {
     const size_t words = ((size_t)(L + 31) / 32 + 2 + 3) / 4 * 4, L4 = (size_t)(L + 3) / 4 * 4;
     return words * 4 + L4 * 9 + 16;

@@ -958,7 +958,7 @@ int read_status(jot_model* m, cudaStream_t st) {
 
 int launch_accept(const AcceptArgs& a, cudaStream_t st, const AcceptParamsInline* inl = nullptr) {
     const size_t smem = accept_smem_bytes(a.L);
-    if (smem > 200 * 1024) return JOT_ERR_SHAPE;
+    if (!accept_length_ok(a.L)) return JOT_ERR_SHAPE;
     if (inl) {
         if (smem > 48 * 1024)
             JOT_CUDA(cudaFuncSetAttribute(accept_freeze_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
