@@ -355,8 +355,8 @@ int run_gemm(const DeviceInfo* di, const CUtensorMap& tmA, const WeightMaps& w, 
             if (norm && p.ldc == p.N && p.N / 8 <= 1024) {
                 int threads = (p.N / 8 + 31) / 32 * 32;      // one 8-element vector per thread up to 512 threads
                 threads = threads > 512 ? 512 : (threads < 64 ? 64 : threads);
-                launch_k(splitk_reduce_norm_kernel, dim3(p.M), dim3(threads), 0, st, scratch, split, p.residual, p.C, p.M,
-                         p.N, norm->gain, norm->out, norm->eps);
+                launch_k(p.N / 8 <= threads ? splitk_reduce_norm_kernel<1> : splitk_reduce_norm_kernel<2>, dim3(p.M), dim3(threads), 0,
+                         st, scratch, split, p.residual, p.C, p.M, p.N, norm->gain, norm->out, norm->eps);
                 norm->done = true;
                 return launch_check();
             }
