@@ -1,4 +1,4 @@
-// The whole transformer body of a small canvas (at most 64 rows) as ONE persistent kernel.
+// The whole transformer body of a small canvas (at most 37 rows on 148 SMs) as ONE persistent kernel.
 //
 // With few rows a pass is a stream of the weights, and as separate launches every projection pays a launch, a pipeline
 // fill, a drain and an epilogue that nothing overlaps (7-10 us each at 32 rows, seven launches a layer; 132 us a layer of the LLaDA-8B shape, 66 us for the bytes; here 107 us).  Here one CTA per
@@ -32,7 +32,7 @@ namespace jot {
 
 constexpr int kBodyThreads = 384;
 constexpr int kBodyWorkers = 256;
-constexpr int kBodyMaxTokens = 64;         // beyond that the separate launches are the faster ones (body_applies)
+constexpr int kBodyMaxTokens = 64;         // what tensor memory is laid out for; body_applies stops earlier
 constexpr int kBodyMaxStages = 8;
 constexpr int kBodyMaxSmem = 226 * 1024;   // dynamic part; the static barriers take the rest of the 227 KB
 constexpr int kBodyWTile = 256 * 128;      // bytes of W per stage: 256 rows x 64 bf16

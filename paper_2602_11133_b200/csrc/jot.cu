@@ -594,17 +594,18 @@ int body_gate_up_rows(int ff, int sms) {
     return (ff + 8 * sms * waves - 1) / (8 * sms * waves) * 8;
 }
 
-// Whether the body of a pass over M rows runs as one launch (body.cuh): few rows, and layers whose weights take HBM longer
-// than the barriers cost.  One launch against separate ones, us for 8 layers and a head: LLaDA-8B shape (436 MB a layer)
-// 1078 / 1193 at 32 rows, 1130 / 1204 at 64, 1223 / 1241 at 96, 1300 / 1270 at 128; Dream-7B shape (466 MB) 1096 / 1160 at 32,
-// 1155 / 1162 at 64, 1200 / 1184 at 80; 2048 columns (103 MB) 561 / 593 at 32, 638 / 612 at 80; 1024 columns (26 MB) 454 / 462
-// at 32, 493 / 478 at 80; 512 columns (6 MB) 394 / 371.  More rows mean more partial sums and more of the step between the
+// Whether the body of a pass over M rows runs as one launch (body.cuh): as few rows as leave each four CTAs in the steps
+// that normalise them (37 on 148 SMs), and layers whose weights take HBM longer than the barriers cost.  One launch against
+// separate ones, us for 8 layers and a head: LLaDA-8B shape (436 MB a layer) 1057 / 1100 at 17 rows, 1079 / 1103 at 32,
+// 1114 / 1110 at 40, 1129 / 1109 at 64; Dream-7B shape (466 MB) 1086 / 1172, 1090 / 1120, 1122 / 1128, 1150 / 1126; 2048 columns
+// (103 MB) 537 / 591, 538 / 580, 562 / 580, 582 / 567; with separate launches of an earlier form 1024 columns (26 MB) were
+// 454 / 462 at 32 rows and 512 columns (6 MB) 394 / 371.  More rows mean more partial sums and longer steps between the
 // projections; small layers have nothing to stream meanwhile.
 bool body_applies(const jot_model* m, int M) {
     const jot_model_config& c = m->cfg;
     const size_t qkv = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, o = (size_t)c.n_q_heads * c.head_dim;
     const size_t layer_bytes = 2 * ((qkv + o) * c.d_model + 3 * (size_t)c.d_ff * c.d_model);
-    return m->body_ok && c.n_layers > 0 && M <= kBodyMaxTokens && layer_bytes >= ((size_t)96 << 20) &&
+    return m->body_ok && c.n_layers > 0 && M <= std::min(m->di->sms / kBodyMaxParts, kBodyMaxTokens) && layer_bytes >= ((size_t)96 << 20) &&
            M * std::max(qkv, (size_t)c.d_model) * 4 <= kSplitKBytes;
 }
 

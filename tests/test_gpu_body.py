@@ -1,5 +1,5 @@
-"""GPU parity of the one-launch transformer body (at most 64 rows of a model with large layers) against the CPU oracle, at
-the sizes where its tiling changes: row counts around the 16-row granularity of the token operand, four CTAs a row or two,
+"""GPU parity of the one-launch transformer body (at most 37 rows of a model with large layers) against the CPU oracle, at
+the sizes where its tiling changes: row counts around the 16-row granularity of the token operand,
 one or two attention items side by side, K ranges, ragged tiles."""
 import pytest
 import torch
@@ -41,10 +41,9 @@ def jot():
     ("hd128", 1, 0, 1),         # one row
     ("hd64", 1, 5, 11),         # 16 rows: one whole granule of the token operand
     ("hd128", 1, 6, 11),        # 17
-    ("hd128", 1, 17, 20),       # 37 rows: the last size with four CTAs a row
-    ("hd128", 2, 9, 10),        # 38 rows: two CTAs a row
-    ("hd64", 8, 3, 5),          # 64 rows of eight short sequences: 320 attention items, side by side
-    ("hd128", 1, 30, 34),       # 64 rows: the last size
+    ("hd128", 1, 10, 22),       # 32 rows
+    ("hd64", 7, 2, 3),          # 35 rows of seven short sequences: 280 attention items, side by side
+    ("hd128", 1, 17, 20),       # 37 rows: the last size
 ])
 def test_step_matches_oracle(jot, weights, name, B, P, G):
     g = GEOMS[name]
@@ -69,8 +68,8 @@ def test_step_matches_oracle(jot, weights, name, B, P, G):
 
 @pytest.mark.parametrize("name,B,P,G,lo,hi", [
     ("hd128", 1, 20, 55, 31, 36),    # five rows at an odd position; the last of three key blocks is ragged
-    ("hd64", 2, 40, 300, 97, 129),   # 64 rows, eleven key blocks: every warp has one, some two
-    ("hd128", 8, 30, 100, 51, 59),   # 64 rows, items side by side: five key blocks over four warps
+    ("hd64", 1, 40, 300, 97, 129),   # 32 rows, eleven key blocks: every warp has one, some two
+    ("hd128", 8, 30, 100, 51, 55),   # 32 rows of 8 sequences, items side by side: five key blocks over four warps
 ])
 def test_block_pass_matches_oracle(jot, weights, name, B, P, G, lo, hi):
     g = GEOMS[name]
