@@ -594,6 +594,11 @@ int body_gate_up_rows(int ff, int sms) {
     return (ff + 8 * sms * waves - 1) / (8 * sms * waves) * 8;
 }
 
+bool body_layers_large(const jot_model_config& c) {
+    const size_t qkv = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, o = (size_t)c.n_q_heads * c.head_dim;
+    return c.n_layers > 0 && 2 * ((qkv + o) * c.d_model + 3 * (size_t)c.d_ff * c.d_model) >= ((size_t)96 << 20);
+}
+
 // Whether the body of a pass over M rows runs as one launch (body.cuh): as few rows as leave each four CTAs in the steps
 // that normalise them (37 on 148 SMs), and layers whose weights take HBM longer than the barriers cost.  One launch against
 // separate ones, us for 8 layers and a head: LLaDA-8B shape (436 MB a layer) 1057 / 1100 at 17 rows, 1079 / 1103 at 32,
@@ -603,10 +608,8 @@ int body_gate_up_rows(int ff, int sms) {
 // projections; small layers have nothing to stream meanwhile.
 bool body_applies(const jot_model* m, int M) {
     const jot_model_config& c = m->cfg;
-    const size_t qkv = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, o = (size_t)c.n_q_heads * c.head_dim;
-    const size_t layer_bytes = 2 * ((qkv + o) * c.d_model + 3 * (size_t)c.d_ff * c.d_model);
-    return m->body_ok && c.n_layers > 0 && M <= std::min(m->di->sms / kBodyMaxParts, kBodyMaxTokens) && layer_bytes >= ((size_t)96 << 20) &&
-           M * std::max(qkv, (size_t)c.d_model) * 4 <= kSplitKBytes;
+    const size_t qkv = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
+    return m->body_ok && M <= std::min(m->di->sms / kBodyMaxParts, kBodyMaxTokens) && M * std::max(qkv, (size_t)c.d_model) * 4 <= kSplitKBytes;
 }
 
 int encode_act_maps(jot_model* m, jot_model::ActMaps* am, int M) {
@@ -1112,14 +1115,14 @@ int jot_init_model(const jot_model_config* cfg, const jot_weights* w, int max_ba
     }
     if ((rc = make_weight_maps(di, &m->wlm, w->lm_head, cfg->vocab, d, false)) != JOT_OK) return fail(rc);
 
-    std::vector<BodyLayer> bl((size_t)cfg->n_layers);
-    for (int l = 0; l < cfg->n_layers; ++l) {
+    std::vector<BodyLayer> bl(body_layers_large(*cfg) ? (size_t)cfg->n_layers : 0);
+    for (size_t l = 0; l < bl.size(); ++l) {
         bl[l].wqkv = m->wqkv[l].m128; bl[l].wo = m->wo[l].m128; bl[l].wdown = m->wdown[l].m128;
         const uint32_t rows = (uint32_t)body_gate_up_rows(cfg->d_ff, di->sms);
         if ((rc = make_map_2d(di, &bl[l].wgu, w->w_gate_up[l], 2 * cfg->d_ff, d, d, rows)) != JOT_OK) return fail(rc);
         bl[l].attn_norm = m->attn_norm[l]; bl[l].mlp_norm = m->mlp_norm[l];
     }
-    {
+    if (!bl.empty()) {
         int dev = 0, coop = 0, per_sm = 0;
         cudaGetDevice(&dev);
         m->body_ok = di->sms <= kBodyMaxCtas && cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
@@ -1139,7 +1142,7 @@ int jot_init_model(const jot_model_config* cfg, const jot_weights* w, int max_ba
     cudaError_t e = cudaMemcpy(m->rope_cs, cs.data(), cs.size() * sizeof(float2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !bl.empty())
         e = cudaMemcpy(m->body_layers, bl.data(), bl.size() * sizeof(BodyLayer), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(m->body_row_sums, 0xff, (size_t)kBodyMaxCtas * kBodyMaxParts * sizeof(unsigned long long));
+    if (e == cudaSuccess && !bl.empty()) e = cudaMemset(m->body_row_sums, 0xff, (size_t)kBodyMaxCtas * kBodyMaxParts * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(m->ctrl, 0, 1024);
     if (e == cudaSuccess) e = cudaMemset(m->hsel, 0, (size_t)m->R_cap * d * 2);
     if (e == cudaSuccess) e = cudaMemset(m->rows, 0, (size_t)m->R_cap * 4);
