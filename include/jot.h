@@ -327,8 +327,7 @@ int jot_gemm_bf16_noalloc(const void* d_A, const void* d_W, const void* d_residu
  * stream around each launch.  jot_profile(m, 1) starts (and clears) the accumulation, jot_profile(m, 0)
  * stops it; jot_profile_read waits for the recorded events and returns, per class, the accumulated
  * device milliseconds and the number of timed spans (host arrays of at least JOT_PROF_CLASSES entries).
- * Classes time single kernels except ROWS (active-row list + final norm / gather, two kernels).  While timing is on, the
- * transformer body of a small canvas, otherwise one launch, runs as the separate kernels the classes name. */
+ * Classes time single kernels except ROWS (active-row list + final norm / gather, two kernels). */
 enum {
     JOT_PROF_EMBED = 0, JOT_PROF_RMSNORM, JOT_PROF_GEMM_QKV, JOT_PROF_ROPE, JOT_PROF_ATTENTION, JOT_PROF_GEMM_O,
     JOT_PROF_GEMM_GATE_UP, JOT_PROF_GEMM_DOWN, JOT_PROF_ROWS, JOT_PROF_LM_HEAD, JOT_PROF_MERGE, JOT_PROF_ACCEPT,

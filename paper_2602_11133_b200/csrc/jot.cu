@@ -17,7 +17,6 @@
 #include "../../include/jot.h"
 #include "accept.cuh"
 #include "attention.cuh"
-#include "body.cuh"
 #include "gemm.cuh"
 #include "gemm2.cuh"
 #include "gemm_slab.cuh"
@@ -431,9 +430,6 @@ struct jot_model {
     float2* partials2;
     int32_t* g_sampled;
     float* splitk;
-    BodyLayer* body_layers;              // every layer's weight maps and gains, for the one-launch body
-    unsigned long long *body_barrier, *body_row_sums;
-    bool body_ok = false;                // one CTA of the body kernel per SM can be resident at once
     int R_cap;
     int32_t* canvas;      // generate: tokens [max_batch * max_seq]
     float *g_top1, *g_top2, *g_sumexp;
@@ -446,20 +442,12 @@ struct jot_model {
     // A-operand maps of the projections for a pass over M rows (rows past M read as zero without memory
     // traffic): one set for the whole canvas, one for the rows of a block
     // (x*: the same buffers as the token operand of the slab kernel, boxes of half an accumulator's tokens)
-    // (b*: and as the token operand of the one-launch body, boxes of every row rounded up to 16)
-    struct ActMaps {
-        int M = -1;
-        bool slab = false, slab_gate_up = false, body = false;
-        CUtensorMap a, attn, act, ba, battn, bact;
-        SlabMaps xa, xattn, xact;
-        int s_qkv = 1, s_o = 1, s_down = 1;      // K ranges of the one-launch body's projections
-    };
+    struct ActMaps { int M = -1; bool slab = false, slab_gate_up = false; CUtensorMap a, attn, act; SlabMaps xa, xattn, xact; };
     ActMaps maps_full, maps_span;
     // block-wise KV cache (caller's memory, optional): per layer the rotated Q/K rows and V^T of the whole canvas
     uint8_t* kv_base = nullptr;
     size_t kv_bytes = 0;
     std::vector<__nv_bfloat16*> kv_qkv, kv_vt;
-    size_t kv_layer_elems = 0;              // from one layer's slice to the next
     std::vector<CUtensorMap> kv_tm_qkv3, kv_tm_vt;
     int kv_map_B = -1, kv_map_L = -1;       // geometry the per-layer maps were encoded for
     int kv_valid_B = -1, kv_valid_L = -1;   // geometry of the last refresh (block passes need one)
@@ -506,7 +494,7 @@ struct ProfScope {
 };
 
 struct Layout {
-    size_t ctrl, rope, h, a, qkv, vt, attn, act, hsel, rows, rows_out, seq_map, partials, partials2, sampled, splitk, body_layers, body_sums, canvas, top1, top2, sumexp, argmax, state, params,
+    size_t ctrl, rope, h, a, qkv, vt, attn, act, hsel, rows, rows_out, seq_map, partials, partials2, sampled, splitk, canvas, top1, top2, sumexp, argmax, state, params,
         total;
 };
 
@@ -550,8 +538,6 @@ Layout make_layout(const jot_model_config* c, int max_batch, int max_seq) {
     l.partials2 = take((size_t)256 * R_cap * sizeof(float2));
     l.sampled = take(M * 4);
     l.splitk = take(kSplitKBytes);
-    l.body_layers = take((size_t)c->n_layers * sizeof(BodyLayer));
-    l.body_sums = take((size_t)kBodyMaxCtas * kBodyMaxParts * sizeof(unsigned long long));
     l.canvas = take(M * 4);
     l.top1 = take(M * 4);
     l.top2 = take(M * 4);
@@ -578,58 +564,12 @@ int encode_activation_maps(jot_model* m, int B, int L) {
     return JOT_OK;
 }
 
-// K ranges per 256-row tile of a projection of the one-launch body: as many as fill the SMs, with at least two k-blocks
-// each and room for the fp32 partial sums.
-int body_pick_split(int M, int N, int K, int sms, int most = kBodyMaxSplit) {
-    const int tiles = (N + 255) / 256, num_kb = (K + 63) / 64;
-    int s = std::min(sms / tiles, most);
-    while (s > 1 && (num_kb / s < 2 || (size_t)s * M * N * 4 > kSplitKBytes)) --s;
-    return s < 1 ? 1 : s;
-}
-
-// Gate rows per tile of its gate/up projection: the fewest that still take no more waves than tiles of 128 would, so that
-// the weights are streamed by as many SMs as there are.
-int body_gate_up_rows(int ff, int sms) {
-    const int waves = (ff + 128 * sms - 1) / (128 * sms);
-    return (ff + 8 * sms * waves - 1) / (8 * sms * waves) * 8;
-}
-
-bool body_layers_large(const jot_model_config& c) {
-    const size_t qkv = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, o = (size_t)c.n_q_heads * c.head_dim;
-    return c.n_layers > 0 && 2 * ((qkv + o) * c.d_model + 3 * (size_t)c.d_ff * c.d_model) >= ((size_t)96 << 20);
-}
-
-// Whether the body of a pass over M rows runs as one launch (body.cuh): as few rows as leave each four CTAs in the steps
-// that normalise them (37 on 148 SMs), and layers whose weights take HBM longer than the barriers cost.  One launch against
-// separate ones, us for 8 layers and a head: LLaDA-8B shape (436 MB a layer) 1057 / 1100 at 17 rows, 1079 / 1103 at 32,
-// 1114 / 1110 at 40, 1129 / 1109 at 64; Dream-7B shape (466 MB) 1086 / 1172, 1090 / 1120, 1122 / 1128, 1150 / 1126; 2048 columns
-// (103 MB) 537 / 591, 538 / 580, 562 / 580, 582 / 567; with separate launches of an earlier form 1024 columns (26 MB) were
-// 454 / 462 at 32 rows and 512 columns (6 MB) 394 / 371.  More rows mean more partial sums and longer steps between the
-// projections; small layers have nothing to stream meanwhile.
-bool body_applies(const jot_model* m, int M) {
-    const jot_model_config& c = m->cfg;
-    const size_t qkv = (size_t)(c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
-    return m->body_ok && M <= std::min(m->di->sms / kBodyMaxParts, kBodyMaxTokens) && M * std::max(qkv, (size_t)c.d_model) * 4 <= kSplitKBytes;
-}
-
 int encode_act_maps(jot_model* m, jot_model::ActMaps* am, int M) {
     if (am->M == M) return JOT_OK;
     const jot_model_config& c = m->cfg;
     JOT_TRY(make_map_2d(m->di, &am->a, m->a, M, c.d_model, c.d_model, 128));
     JOT_TRY(make_map_2d(m->di, &am->attn, m->attn, M, c.n_q_heads * c.head_dim, c.n_q_heads * c.head_dim, 128));
     JOT_TRY(make_map_2d(m->di, &am->act, m->act, M, c.d_ff, c.d_ff, 128));
-    am->body = body_applies(m, M);
-    if (am->body) {
-        const uint32_t box = (uint32_t)(M + 15) / 16 * 16;
-        const int qkv_cols = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim, o_cols = c.n_q_heads * c.head_dim;
-        JOT_TRY(make_map_2d(m->di, &am->ba, m->a, M, c.d_model, c.d_model, box));
-        JOT_TRY(make_map_2d(m->di, &am->battn, m->attn, M, o_cols, o_cols, box));
-        JOT_TRY(make_map_2d(m->di, &am->bact, m->act, M, c.d_ff, c.d_ff, box));
-        // (QKV: more than four ranges cost the step that adds them as much as they save)
-        am->s_qkv = body_pick_split(M, qkv_cols, c.d_model, m->di->sms, 4);
-        am->s_o = body_pick_split(M, c.d_model, o_cols, m->di->sms);
-        am->s_down = body_pick_split(M, c.d_model, c.d_ff, m->di->sms);
-    }
     am->slab = M <= kSlabPreferTokens;
     am->slab_gate_up = (M > 128 && M <= kSlabGateUpTokens) ||
                        ((2 * c.d_ff) % 256 == 0 &&
@@ -768,69 +708,12 @@ struct ActiveRows {
     int max_rows;                  // at most this many
 };
 
-// The body of a small canvas as one cooperative launch, from tokens to the normalised active rows in m->hsel.
-int launch_body(jot_model* m, const jot_model::ActMaps& am, const int32_t* d_tokens, int B, int L, cudaStream_t st,
-                const int32_t* seq_map, int Lr, int pos0, bool cached, const ActiveRows& ar) {
-    const jot_model_config& c = m->cfg;
-    BodyParams p{};
-    p.layers = m->body_layers; p.n_layers = c.n_layers;
-    p.M = B * Lr; p.n_tok = (p.M + 15) / 16 * 16;
-    p.B = B; p.L = L; p.Lp = (int)align_up((size_t)L, 8); p.rows_per_seq = Lr; p.pos0 = pos0;
-    p.d = c.d_model; p.ff = c.d_ff; p.nq = c.n_q_heads; p.nkv = c.n_kv_heads; p.hd = c.head_dim; p.vocab = c.vocab;
-    p.eps = c.rms_eps; p.scale_log2e = 1.4426950408889634f / sqrtf((float)c.head_dim);
-    p.s_qkv = am.s_qkv; p.s_o = am.s_o; p.s_down = am.s_down;
-    p.gu_rows = body_gate_up_rows(c.d_ff, m->di->sms);
-    p.h = m->h; p.a = m->a; p.attn = m->attn; p.act = m->act; p.hsel = m->hsel;
-    p.qkv = cached ? m->kv_qkv[0] : m->qkv;
-    p.vt = cached ? m->kv_vt[0] : m->vt;
-    p.qkv_stride = p.vt_stride = cached ? m->kv_layer_elems : 0;
-    p.rope_cs = m->rope_cs; p.partial = m->splitk; p.tokens = d_tokens; p.embed = m->embed; p.final_norm = m->final_norm;
-    p.seq_map = seq_map; p.mask_id = c.mask_id; p.blk_lo = ar.blk_lo; p.blk_hi = ar.blk_hi; p.state = ar.state;
-    p.P = ar.P; p.block_len = ar.block_len; p.n_blocks = ar.n_blocks;
-    p.rows = m->rows; p.rows_out = m->rows_out; p.d_R = m->ctrl + 1;
-    {
-        // rounds of 32-key blocks a warp goes through, with all warps on one item or half of them; a tie means fewer exchanges
-        auto up = [](int a, int b) { return (a + b - 1) / b; };
-        const int items = B * c.n_q_heads * up(Lr, kBodyQT), blocks = up(L, 32), sms = m->di->sms;
-        p.attn_pairs = items > sms && up(items, 2 * sms) * up(blocks, 4) <= up(items, sms) * up(blocks, 8);
-    }
-    p.parts = 1;
-    while (p.parts < kBodyMaxParts && p.M * p.parts * 2 <= m->di->sms) p.parts *= 2;
-    p.row_sums = m->body_row_sums; p.barrier = m->body_barrier; p.status = m->ctrl;
-    p.stage_bytes = kBodyWTile + p.n_tok * 128;
-    const int work = body_work_bytes(c.head_dim, c.d_model);
-    p.stages = std::min(kBodyMaxStages, (kBodyMaxSmem - 1024 - work) / p.stage_bytes);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)m->di->sms);
-    cfg.blockDim = dim3(kBodyThreads);
-    cfg.dynamicSmemBytes = (size_t)(p.stages * p.stage_bytes + work + 1024);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, body_kernel, p, am.ba, am.battn, am.bact);
-    return launch_check();
-}
-
 // Tokens [B, L] -> the list of active rows (m->rows, m->rows_out, their count in m->ctrl[1]) and their final-normalised
-// hidden states in m->hsel.  While kernels are being timed one by one (jot_profile) the body runs as separate launches
-// at every size.
+// hidden states in m->hsel.
 int forward_to_head(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStream_t st, const int32_t* seq_map,
                     const FwdSpan* span, const ActiveRows& ar) {
     const jot_model_config& c = m->cfg;
     const int Lr = span ? span->Lr : L, pos0 = span ? span->pos0 : 0;
-    if (!m->profiling && body_applies(m, B * Lr)) {
-        jot_model::ActMaps& am = (Lr == L) ? m->maps_full : m->maps_span;
-        JOT_TRY(encode_activation_maps(m, B, L));
-        JOT_TRY(encode_act_maps(m, &am, B * Lr));
-        const bool cached = span && span->use_cache;
-        if (cached) JOT_TRY(encode_kv_maps(m, B, L));
-        const int rc = launch_body(m, am, d_tokens, B, L, st, seq_map, Lr, pos0, cached, ar);
-        if (rc != JOT_ERR_CUDA || g_last_cuda_error != (int)cudaErrorCooperativeLaunchTooLarge) return rc;
-        m->body_ok = false;                    // a context with a part of the SMs: its CTAs cannot all be resident
-    }
     JOT_TRY(forward_body(m, d_tokens, B, L, st, seq_map, span));
     ProfScope ps(m, JOT_PROF_ROWS, st);
     launch_k(build_rows_kernel, dim3(1), dim3(1024), 0, st, d_tokens, B, L, c.mask_id, ar.blk_lo, ar.blk_hi, ar.state, ar.P,
@@ -1078,9 +961,6 @@ int jot_init_model(const jot_model_config* cfg, const jot_weights* w, int max_ba
     m->partials2 = (float2*)(base + lay.partials2);
     m->g_sampled = (int32_t*)(base + lay.sampled);
     m->splitk = (float*)(base + lay.splitk);
-    m->body_layers = (BodyLayer*)(base + lay.body_layers);
-    m->body_row_sums = (unsigned long long*)(base + lay.body_sums);
-    m->body_barrier = (unsigned long long*)(base + lay.ctrl + 512);
     m->R_cap = (int)align_up((size_t)max_batch * max_seq, 128);
     m->canvas = (int32_t*)(base + lay.canvas);
     m->g_top1 = (float*)(base + lay.top1);
@@ -1115,23 +995,6 @@ int jot_init_model(const jot_model_config* cfg, const jot_weights* w, int max_ba
     }
     if ((rc = make_weight_maps(di, &m->wlm, w->lm_head, cfg->vocab, d, false)) != JOT_OK) return fail(rc);
 
-    std::vector<BodyLayer> bl(body_layers_large(*cfg) ? (size_t)cfg->n_layers : 0);
-    for (size_t l = 0; l < bl.size(); ++l) {
-        bl[l].wqkv = m->wqkv[l].m128; bl[l].wo = m->wo[l].m128; bl[l].wdown = m->wdown[l].m128;
-        const uint32_t rows = (uint32_t)body_gate_up_rows(cfg->d_ff, di->sms);
-        if ((rc = make_map_2d(di, &bl[l].wgu, w->w_gate_up[l], 2 * cfg->d_ff, d, d, rows)) != JOT_OK) return fail(rc);
-        bl[l].attn_norm = m->attn_norm[l]; bl[l].mlp_norm = m->mlp_norm[l];
-    }
-    if (!bl.empty()) {
-        int dev = 0, coop = 0, per_sm = 0;
-        cudaGetDevice(&dev);
-        m->body_ok = di->sms <= kBodyMaxCtas && cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-                     cudaFuncSetAttribute(body_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBodyMaxSmem) == cudaSuccess &&
-                     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, body_kernel, kBodyThreads, kBodyMaxSmem) == cudaSuccess &&
-                     per_sm > 0;
-        cudaGetLastError();
-    }
-
     // tables: cos/sin of pos * theta^(-2j/hd), evaluated in double on the host once
     std::vector<float2> cs((size_t)max_seq * (hd / 2));
     for (int pos = 0; pos < max_seq; ++pos)
@@ -1140,9 +1003,6 @@ int jot_init_model(const jot_model_config* cfg, const jot_weights* w, int max_ba
             cs[(size_t)pos * (hd / 2) + j] = make_float2((float)std::cos(ang), (float)std::sin(ang));
         }
     cudaError_t e = cudaMemcpy(m->rope_cs, cs.data(), cs.size() * sizeof(float2), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !bl.empty())
-        e = cudaMemcpy(m->body_layers, bl.data(), bl.size() * sizeof(BodyLayer), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !bl.empty()) e = cudaMemset(m->body_row_sums, 0xff, (size_t)kBodyMaxCtas * kBodyMaxParts * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(m->ctrl, 0, 1024);
     if (e == cudaSuccess) e = cudaMemset(m->hsel, 0, (size_t)m->R_cap * d * 2);
     if (e == cudaSuccess) e = cudaMemset(m->rows, 0, (size_t)m->R_cap * 4);
@@ -1259,7 +1119,6 @@ int jot_attach_kv_cache(jot_model* m, void* d_cache, size_t bytes) {
         m->kv_qkv[l] = (__nv_bfloat16*)base;
         m->kv_vt[l] = (__nv_bfloat16*)(base + vt_off);
     }
-    m->kv_layer_elems = per_layer / sizeof(__nv_bfloat16);
     m->kv_base = (uint8_t*)d_cache;
     m->kv_bytes = bytes;
     return JOT_OK;
