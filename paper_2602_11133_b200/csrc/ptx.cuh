@@ -235,15 +235,17 @@ __device__ __forceinline__ void tmem_ld_wait_regs(float* v) {
         : "memory");
 }
 
-// silu(g) * u = g / (1 + exp(-g)) * u.  The quotient by a denominator in [1, FLT_MAX]: a reciprocal estimate and one residual
-// correction (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990), without the
-// range checks of a general division, whose branches keep a loop over many elements from overlapping them.
+// silu(g) * u = g / (1 + exp(-g)) * u.  The quotient: a reciprocal estimate and one residual correction (Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor", 1990), without the range checks of a general
+// division, whose branches keep a loop over many elements from overlapping them.  The estimate keeps subnormals: above 2^126
+// (gates below -87.3) they are what the reciprocal is.  Of all 2^32 gates three differ from the division, by one ulp; an
+// estimate that flushes subnormals made the quotient 0 there, at the same time per step (993 rows: 13.21 / 13.30 ms).
 __device__ __forceinline__ float silu_mul(float g, float u) {
-    const float den = fminf(1.f + __expf(-g), 3.402823466e38f);
+    const float den = 1.f + __expf(-g);
     float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(den));
+    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(den));
     const float q = g * y, r = fmaf(-q, den, g);
-    return (r == r ? fmaf(r, y, q) : q) * u;            // (g infinite: the residual is not a number, the quotient is right)
+    return (r == r ? fmaf(r, y, q) : q) * u;            // no residual where g or the denominator is infinite: q is the quotient there
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
