@@ -5,6 +5,7 @@
 // the argmax token into every chosen position (Algorithm 1).
 #pragma once
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <stdint.h>
 
 #include "pdl.cuh"
@@ -80,11 +81,12 @@ __device__ __forceinline__ AcceptParamsDev accept_pick_params(const AcceptArgs& 
 }
 
 // The kernel is a chain of memory round trips and barriers over a few hundred numbers, so it is kept short: everything a
-// decision reads is requested before the canvas has arrived, thread t looks after position lo + t of the block (no list of
-// candidates is built), and the ranks are counted by all threads together: 8.3 -> 5.8 us for a block of 32 in a canvas of 384
-// as ncu times it.
-// Dynamic shared memory: resolved bitmap words; per position of the block its rank, sum-exp (not a number where there is
-// nothing to rank: no comparison with it holds) and flags.
+// decision reads is requested before the canvas has arrived, thread t looks after position lo + t of the block, and the ranks
+// are counted by all threads together.  What is ranked stands in a list of its own: a long block with few positions left must
+// not pay for the ones that are decided.  Call after call in a graph, with 5 % / all of the positions masked: 2.8 / 2.8 us for a
+// block of 32 in a canvas of 384, 3.8 / 11.3 for 512 in 704, 31 / 1937 for 8192 (comparing with every position of the block: 3.9 /
+// 3.9, 16 / 16, 2281 / 2675).
+// Dynamic shared memory: resolved bitmap words; the list of (sum-exp, position) to rank; per position of the block its flags.
 template <bool INLINE>
 __global__ void __launch_bounds__(kAcceptThreads)
 accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename AcceptInlineArg<INLINE>::type inl) {
@@ -95,11 +97,12 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
     const int n_words = (L + 31) / 32;
     uint32_t* res_bits = sh;                                   // [n_words + 2] resolved bitmap (padded)
     const int L4 = (L + 3) & ~3;
-    float* pos_S = reinterpret_cast<float*>(sh + ((n_words + 2 + 3) & ~3));       // [L4] 16-byte aligned
-    int* rank = reinterpret_cast<int*>(pos_S + L4);                               // [L4]
-    uint8_t* flag = reinterpret_cast<uint8_t*>(rank + L4);                        // [L4] bit0 exit, bit1 schedule
+    uint64_t* keys = reinterpret_cast<uint64_t*>(sh + ((n_words + 2 + 3) & ~3));  // [L4] 16-byte aligned, in any order
+    uint8_t* flag = reinterpret_cast<uint8_t*>(keys + L4);                        // [L4] bit0 exit, bit1 schedule, bit2 ranks first
     __shared__ float gpow[kMaxD + 1];
-    __shared__ int n_cand_sh, n_final_sh;
+    __shared__ int rank[kAcceptThreads];                       // of the positions of a block no longer than this
+    __shared__ uint32_t counts_sh;                             // entries of the list; candidates in the upper half (both below 2^15)
+    __shared__ int n_final_sh;
     __shared__ float inv_wmax;
     __shared__ float ratio_sums[kAcceptThreads / 32], gap_sums[kAcceptThreads / 32];
 
@@ -145,7 +148,7 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
             sum += g;
         }
         inv_wmax = 1.f / (2.f * sum);
-        n_cand_sh = 0;
+        counts_sh = 0;
         n_final_sh = 0;
     }
     for (int w = n_words + tid; w < n_words + 2; w += blockDim.x) res_bits[w] = 0;
@@ -164,24 +167,32 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
     __syncthreads();
 
     // per candidate (masked position of the block): ratio, threshold, early-exit decision
-    const float none = __int_as_float(0x7fffffff);
     float r_sum = 0.f, gap_sum = 0.f;
-    int mine = 0;
-    for (int c = tid; c < ((n_pos + 3) & ~3); c += kAcceptThreads) {
-        const int i = lo + c;
-        float S = none;
+    float m1_next = m1_0, m2_next = m2_0, S_next = S_0;
+    for (int base = 0; base < n_pos; base += kAcceptThreads) {
+        const int c = base + tid, i = lo + c;
+        const float m1 = m1_next, m2 = m2_next, S = S_next;
+        if (c + kAcceptThreads < n_pos) {                      // the next 256 positions' statistics are on their way meanwhile
+            m1_next = a.top1[row + i + kAcceptThreads];
+            m2_next = a.top2[row + i + kAcceptThreads];
+            S_next = a.sumexp[row + i + kAcceptThreads];
+        }
+        const bool cand = c < n_pos && !((res_bits[i >> 5] >> (i & 31)) & 1u);
+        bool listed = false;
         uint8_t f = 0;
-        if (c < n_pos && !((res_bits[i >> 5] >> (i & 31)) & 1u)) {
-            const float m1 = c < kAcceptThreads ? m1_0 : a.top1[row + i], m2 = c < kAcceptThreads ? m2_0 : a.top2[row + i];
-            S = c < kAcceptThreads ? S_0 : a.sumexp[row + i];
+        if (cand) {
             // Eq. 4 with p1 = 1/S, p2 = exp(m2 - m1)/S:  r = 1 / (exp(m2 - m1) + eps * S)
             const float r = 1.f / (expf(m2 - m1) + prm.eps * S);
-            // Eq. 5: resolved neighbours at distance 1..D on both sides, read from the bitmap
+            // Eq. 5: resolved neighbours at distance 1..D <= 32 on both sides, 32 bits of the bitmap each (zero past its ends)
+            const int iw = i >> 5, rw = (i + 1) >> 5;
+            const uint32_t left = __funnelshift_r(iw ? res_bits[iw - 1] : 0u, res_bits[iw], i & 31);      // bit 32 - d: i - d
+            const uint32_t right = __funnelshift_r(res_bits[rw], res_bits[rw + 1], (i + 1) & 31);         // bit d - 1: i + d
             float w = 0.f;
+#pragma unroll 4
             for (int d = 1; d <= prm.D; ++d) {
-                int jl = i - d, jr = i + d;
-                if (jl >= 0 && ((res_bits[jl >> 5] >> (jl & 31)) & 1u)) w += gpow[d];
-                if (jr < L && ((res_bits[jr >> 5] >> (jr & 31)) & 1u)) w += gpow[d];
+                const float g = gpow[d];
+                w += (left >> (32 - d)) & 1u ? g : 0.f;
+                w += (right >> (d - 1)) & 1u ? g : 0.f;
             }
             const float phi = fminf(1.f, w * inv_wmax);                        // Eq. 6
             const float tau = prm.tau_max - (prm.tau_max - prm.tau_min) * phi; // Eq. 7
@@ -190,14 +201,24 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
             // Eq. 8; or the fixed probability gate the paper contrasts it with (p1 = 1/S, no spatial modulation)
             // (the global early-commit gate decides for all candidates together, after the sum below)
             f = (prm.gate == 1 ? (1.f / S >= prm.prob_threshold) : (prm.gate == 2 ? false : r >= tau)) ? 1 : 0;
-            ++mine;
-            if (prm.schedule_after_exit && f && prm.gate != 2) S = none;         // the schedule ranks what is left
+            listed = !(prm.schedule_after_exit && f);                            // the schedule ranks what is left
+            if (listed && !(S == S)) {                                           // a sum that is no number ranks first, ahead of no one
+                f |= 4;
+                listed = false;
+            }
         }
-        pos_S[c] = S;
-        rank[c] = 0;
-        flag[c] = f;
+        if (base == 0) rank[tid] = listed ? 0 : INT_MAX;
+        if (c < n_pos) flag[c] = f;
+        const uint32_t in_list = __ballot_sync(0xffffffffu, listed), all = __ballot_sync(0xffffffffu, cand);
+        uint32_t at = 0;
+        if ((tid & 31) == 0 && all) at = atomicAdd(&counts_sh, (uint32_t)__popc(all) << 16 | (uint32_t)__popc(in_list));
+        at = (__shfl_sync(0xffffffffu, at, 0) & 0xffffu) + __popc(in_list & ((1u << (tid & 31)) - 1u));
+        if (listed) {
+            // ordered like (S, position); -0 counts as 0
+            const uint32_t bits = __float_as_uint(S + 0.f);
+            keys[at] = (uint64_t)(bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u)) << 32 | (uint32_t)c;
+        }
     }
-    if (mine) atomicAdd(&n_cand_sh, mine);
     if (prm.gate == 2) {                                       // fixed-order tree: the same sum on every run
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) gap_sum += __shfl_xor_sync(0xffffffffu, gap_sum, o);
@@ -209,7 +230,7 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
         if ((tid & 31) == 0) ratio_sums[tid >> 5] = r_sum;
     }
     __syncthreads();
-    const int n_cand = n_cand_sh;
+    const int n_cand = counts_sh >> 16, n_list = counts_sh & 0xffffu;
     auto is_cand = [&](int c) { return !((res_bits[(lo + c) >> 5] >> ((lo + c) & 31)) & 1u); };
     if (a.state && prm.schedule == 1) {
         // adaptive schedule: the share of what is still masked that keeps the block on pace to end with its last step
@@ -217,41 +238,35 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
         k = (n_cand + steps_left - 1) / steps_left;
     }
 
+    bool all_exit = false;
     if (prm.gate == 2 && n_cand > 0) {
         // global early commit: every candidate exits when the mean top-2 logit gap clears the threshold
         float t = 0.f;
         for (int w = 0; w < kAcceptThreads / 32; ++w) t += gap_sums[w];
-        if (t / (float)n_cand >= prm.gap_threshold)
-            for (int c = tid; c < n_pos; c += blockDim.x)
-                if (is_cand(c)) {
-                    flag[c] = 1;
-                    if (prm.schedule_after_exit) pos_S[c] = none;
-                }
-        __syncthreads();                                       // the schedule below reads other threads' values
+        all_exit = t / (float)n_cand >= prm.gap_threshold;
     }
 
     // transfer schedule: the k candidates with the largest p1 = 1/S, i.e. the smallest S; equal S
-    // resolves to the lower position.  Rank by counting: W threads take a position each, 256 / W of them share its
+    // resolves to the lower position.  Rank by counting: W threads take an entry each, 256 / W of them share its
     // comparisons.
-    const int k_eff = min(k, n_cand);
+    const int k_eff = all_exit && prm.schedule_after_exit ? 0 : min(k, n_cand);
+    const bool short_block = n_pos <= kAcceptThreads;
     if (k_eff > 0) {
         int W = 32;
-        while (W < n_pos && W < kAcceptThreads) W <<= 1;
-        const int share = kAcceptThreads / W, q = tid / W;
-        const int n4 = (n_pos + 3) >> 2, o_lo = n4 * q / share, o_hi = n4 * (q + 1) / share;
-        for (int c = tid % W; c < n_pos; c += W) {
-            const float Sc = pos_S[c];
-            if (!(Sc == Sc)) continue;                         // nothing to rank here; a sum that is no number ranks first
+        while (W < (short_block ? n_list : kAcceptThreads) && W < kAcceptThreads) W <<= 1;
+        const int share = kAcceptThreads / W, q = tid / W, pairs = n_list >> 1;
+        const int o_lo = pairs * q / share, o_hi = pairs * (q + 1) / share;
+        for (int e = tid % W; e < n_list; e += W) {
+            const uint64_t key = keys[e];
             int before = 0;
             for (int o = o_lo; o < o_hi; ++o) {
-                const float4 v = reinterpret_cast<const float4*>(pos_S)[o];
-                const int o0 = o * 4;
-                before += (v.x < Sc) || (v.x == Sc && o0 < c);
-                before += (v.y < Sc) || (v.y == Sc && o0 + 1 < c);
-                before += (v.z < Sc) || (v.z == Sc && o0 + 2 < c);
-                before += (v.w < Sc) || (v.w == Sc && o0 + 3 < c);
+                const ulonglong2 v = reinterpret_cast<const ulonglong2*>(keys)[o];
+                before += (v.x < key) + (v.y < key);
             }
-            atomicAdd(&rank[c], before);
+            if ((n_list & 1) && q == share - 1) before += keys[n_list - 1] < key;
+            const int c = (int)(uint32_t)key;
+            if (short_block) atomicAdd(&rank[c], before);
+            else if (before < k_eff) flag[c] |= 2;
         }
         __syncthreads();
     }
@@ -259,9 +274,9 @@ accept_freeze_kernel(const AcceptArgs a, const __grid_constant__ typename Accept
     // freeze: chosen candidates receive their argmax; everything else is left untouched
     int my_final = 0;
     for (int c = tid; c < n_pos; c += blockDim.x) {
-        const uint8_t exited = flag[c];
-        const bool ranked = k_eff > 0 && is_cand(c) && !(prm.schedule_after_exit && (exited & 1));
-        const uint8_t f = exited | ((ranked && rank[c] < k_eff) ? 2 : 0);
+        uint8_t f = flag[c] | (all_exit && is_cand(c) ? 1 : 0);
+        if (k_eff > 0 && ((f & 4) || (short_block && rank[c] < k_eff))) f |= 2;
+        f &= 3;
         if (f) {
             const int i = lo + c;
             const size_t gi = row + i;
