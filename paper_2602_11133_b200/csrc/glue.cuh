@@ -63,55 +63,71 @@ __global__ void embed_kernel(const int32_t* __restrict__ tokens, const __nv_bflo
 
 // out[r, :] = bf16( x[src_row, :] * rsqrt(mean(x^2) + eps) * gain ),  src_row = rows ? rows[r] : r.
 // With `rows`, only r < *d_R is processed (final norm + compaction of the active rows).
-// One CTA per output row; d multiple of 8 and d/8 <= 8 * blockDim.x.
-__global__ void rmsnorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gain,
-                               __nv_bfloat16* __restrict__ out, int d, float eps, const int32_t* __restrict__ rows,
-                               const int32_t* __restrict__ d_R) {
+// One row per CTA at a time, MAXV 8-element vectors per thread; d multiple of 8 and d/8 <= MAXV * blockDim.x.  Bound by the
+// latency of a row (load, block sum, store), so by how many rows an SM has in flight: a CTA takes every gridDim.x-th row and
+// requests the next one before it reduces the present one, and MAXV is no larger than d asks for.  11264 rows of 4096: 80 -> 44 us
+// (184 MB: 2.3 -> 4.2 TB/s) against one CTA per row with room for 8 vectors a thread; 32 rows 8.7 -> 6.7 us (the gain vector no
+// longer comes after the sum).
+template <int MAXV>
+__global__ void __launch_bounds__(256, MAXV <= 2 ? 4 : (MAXV <= 4 ? 2 : 1))
+rmsnorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ out, int d,
+               float eps, int n_rows, const int32_t* __restrict__ rows, const int32_t* __restrict__ d_R) {
     grid_launch_dependents();
-    grid_dependency_wait();
     __shared__ float scratch[33];
-    const int r = blockIdx.x;
-    int src = r;
-    if (rows) {
-        if (r >= *d_R) return;
-        src = rows[r];
-    }
-    const uint4* xin = reinterpret_cast<const uint4*>(x + (size_t)src * d);
     const int nvec = d / 8;
-    constexpr int MAXV = 8;
-    uint4 buf[MAXV];
-    float ss = 0.f;
+    uint4 gv[MAXV], buf[MAXV], next[MAXV];
+    // the gain is a weight, nobody's output: it is requested before the wait on the preceding kernel
 #pragma unroll
     for (int t = 0; t < MAXV; ++t) {
-        int i = threadIdx.x + t * blockDim.x;
-        if (i < nvec) {
-            buf[t] = xin[i];
-            const __nv_bfloat162* b2 = reinterpret_cast<const __nv_bfloat162*>(&buf[t]);
+        const int i = threadIdx.x + t * blockDim.x;
+        if (i < nvec) gv[t] = reinterpret_cast<const uint4*>(gain)[i];
+    }
+    grid_dependency_wait();
+    const int R = rows ? *d_R : n_rows;
+    auto request = [&](int r) {
+        const uint4* xin = reinterpret_cast<const uint4*>(x + (size_t)(rows ? rows[r] : r) * d);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                float2 f = __bfloat1622float2(b2[j]);
-                ss += f.x * f.x + f.y * f.y;
+        for (int t = 0; t < MAXV; ++t) {
+            const int i = threadIdx.x + t * blockDim.x;
+            if (i < nvec) next[t] = xin[i];
+        }
+    };
+    int r = blockIdx.x;
+    if (r < R) request(r);
+    for (; r < R; r += gridDim.x) {
+#pragma unroll
+        for (int t = 0; t < MAXV; ++t) buf[t] = next[t];
+        if (r + (int)gridDim.x < R) request(r + gridDim.x);
+        float ss = 0.f;
+#pragma unroll
+        for (int t = 0; t < MAXV; ++t) {
+            if (threadIdx.x + t * blockDim.x < nvec) {
+                const __nv_bfloat162* b2 = reinterpret_cast<const __nv_bfloat162*>(&buf[t]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 f = __bfloat1622float2(b2[j]);
+                    ss += f.x * f.x + f.y * f.y;
+                }
             }
         }
-    }
-    ss = block_sum(ss, scratch);
-    const float inv = rsqrtf(ss / (float)d + eps);
-    const uint4* g4 = reinterpret_cast<const uint4*>(gain);
-    uint4* o4 = reinterpret_cast<uint4*>(out + (size_t)r * d);
+        ss = block_sum(ss, scratch);
+        const float inv = rsqrtf(ss / (float)d + eps);
+        uint4* o4 = reinterpret_cast<uint4*>(out + (size_t)r * d);
 #pragma unroll
-    for (int t = 0; t < MAXV; ++t) {
-        int i = threadIdx.x + t * blockDim.x;
-        if (i < nvec) {
-            uint4 gv = g4[i], ov;
-            const __nv_bfloat162* b2 = reinterpret_cast<const __nv_bfloat162*>(&buf[t]);
-            const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&gv);
-            __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&ov);
+        for (int t = 0; t < MAXV; ++t) {
+            const int i = threadIdx.x + t * blockDim.x;
+            if (i < nvec) {
+                uint4 ov;
+                const __nv_bfloat162* b2 = reinterpret_cast<const __nv_bfloat162*>(&buf[t]);
+                const __nv_bfloat162* g2 = reinterpret_cast<const __nv_bfloat162*>(&gv[t]);
+                __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&ov);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                float2 f = __bfloat1622float2(b2[j]), g = __bfloat1622float2(g2[j]);
-                o2[j] = __floats2bfloat162_rn(f.x * inv * g.x, f.y * inv * g.y);
+                for (int j = 0; j < 4; ++j) {
+                    const float2 f = __bfloat1622float2(b2[j]), g = __bfloat1622float2(g2[j]);
+                    o2[j] = __floats2bfloat162_rn(f.x * inv * g.x, f.y * inv * g.y);
+                }
+                o4[i] = ov;
             }
-            o4[i] = ov;
         }
     }
 }

@@ -405,6 +405,17 @@ int launch_attention_t(const AttnParams& p, const CUtensorMap& tq, const CUtenso
     return launch_check();
 }
 
+// Rows of d elements (at most 16384): as few vectors per thread as d allows, CTAs for as many rows as run side by side.
+int launch_rmsnorm(const DeviceInfo* di, const __nv_bfloat16* x, const __nv_bfloat16* gain, __nv_bfloat16* out, int d, float eps, int n_rows,
+                   const int32_t* rows, const int32_t* d_R, cudaStream_t st) {
+    const int nvec = d / 8, maxv = nvec <= 512 ? 2 : (nvec <= 1024 ? 4 : 8), per_sm = maxv == 2 ? 4 : (maxv == 4 ? 2 : 1);
+    const dim3 grid((unsigned)std::min(n_rows, per_sm * di->sms)), block(256);
+    if (maxv == 2) launch_k(rmsnorm_kernel<2>, grid, block, 0, st, x, gain, out, d, eps, n_rows, rows, d_R);
+    else if (maxv == 4) launch_k(rmsnorm_kernel<4>, grid, block, 0, st, x, gain, out, d, eps, n_rows, rows, d_R);
+    else launch_k(rmsnorm_kernel<8>, grid, block, 0, st, x, gain, out, d, eps, n_rows, rows, d_R);
+    return launch_check();
+}
+
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 }  // namespace
@@ -640,8 +651,7 @@ int forward_body(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStream
     for (int l = 0; l < c.n_layers; ++l) {
         if (!norm_ready) {
             ProfScope ps(m, JOT_PROF_RMSNORM, st);
-            launch_k(rmsnorm_kernel, dim3(M), dim3(256), 0, st, m->h, m->attn_norm[l], m->a, d, c.rms_eps, nullptr, nullptr);
-            JOT_TRY(launch_check());
+            JOT_TRY(launch_rmsnorm(m->di, m->h, m->attn_norm[l], m->a, d, c.rms_eps, M, nullptr, nullptr, st));
         }
         GemmParams p{};
         p.M = M; p.N = qkv_cols; p.K = d; p.C = cached ? m->kv_qkv[l] : m->qkv; p.ldc = qkv_cols; p.status = status;
@@ -675,8 +685,7 @@ int forward_body(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStream
         }
         if (!norm_ready) {
             ProfScope ps(m, JOT_PROF_RMSNORM, st);
-            launch_k(rmsnorm_kernel, dim3(M), dim3(256), 0, st, m->h, m->mlp_norm[l], m->a, d, c.rms_eps, nullptr, nullptr);
-            JOT_TRY(launch_check());
+            JOT_TRY(launch_rmsnorm(m->di, m->h, m->mlp_norm[l], m->a, d, c.rms_eps, M, nullptr, nullptr, st));
         }
         p = GemmParams{};
         p.M = M; p.N = 2 * c.d_ff; p.K = d; p.C = m->act; p.ldc = c.d_ff; p.status = status;
@@ -719,9 +728,7 @@ int forward_to_head(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStr
     launch_k(build_rows_kernel, dim3(1), dim3(1024), 0, st, d_tokens, B, L, c.mask_id, ar.blk_lo, ar.blk_hi, ar.state, ar.P,
              ar.block_len, ar.n_blocks, seq_map, m->rows, m->rows_out, m->ctrl + 1, Lr, pos0);
     JOT_TRY(launch_check());
-    launch_k(rmsnorm_kernel, dim3(std::max(1, ar.max_rows)), dim3(256), 0, st, m->h, m->final_norm, m->hsel, c.d_model,
-             c.rms_eps, m->rows, m->ctrl + 1);
-    return launch_check();
+    return launch_rmsnorm(m->di, m->h, m->final_norm, m->hsel, c.d_model, c.rms_eps, std::max(1, ar.max_rows), m->rows, m->ctrl + 1, st);
 }
 
 // hsel (active rows, already gathered) -> merged statistics scattered to the [B, L] outputs
