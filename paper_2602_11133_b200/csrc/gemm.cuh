@@ -69,6 +69,8 @@ struct GemmParams {
     int step_value;               // step_value); b = flat canvas index / L
     float2* partials2;            // [chunks][R_pad] (best perturbed score, bitcast token)
     int R_pad;                    // row capacity of one chunk of partials (multiple of 128)
+    // CTA-pair kernel only (gemm2.cuh): W columns of a tile, row-block pairs of a band of tiles
+    int bn, band;
     // slab kernel only (gemm_slab.cuh): first pair-slab of the launch and pairs per cluster (K ranges)
     int slab0, slab_split;
 };
@@ -129,25 +131,28 @@ __device__ __forceinline__ void stats_row_init(const GemmParams& p, int row, Sta
 }
 
 // Epilogue of one 128 x BN accumulator tile: the calling thread owns output row `row` (TMEM lane) and reads
-// it 32 columns at a time from tensor memory at `t_acc`.  Shared by the one-CTA and the CTA-pair kernels.
+// it 32 columns at a time from tensor memory at `t_acc`.  Shared by the one-CTA and the CTA-pair kernels.  The tile has
+// bn <= BN columns of W: a multiple of 16 with EPI_STORE, of 32 with EPI_SWIGLU (half of them gate columns, half up), BN with
+// the others.  Where 32 is no divisor the last read takes in accumulator columns next to the tile's, which are not used.
 template <int BN, int EPI>
 __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t t_acc, int row, int n_blk, int ks,
-                                              int n_out, StatsRow& st, float* stg = nullptr) {
+                                              int n_out, StatsRow& st, float* stg = nullptr, int bn = BN) {
     constexpr float L2E = 1.4426950408889634f;
     (void)L2E; (void)ks; (void)n_out; (void)st;
     if (EPI == EPI_STORE) {
+        const int col_end = min(p.N, n_blk * bn + bn);
 #pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
+        for (int c = 0; c * 32 < bn; ++c) {
             float v[32];
             tmem_ld32(t_acc + c * 32, v);
             tmem_ld_wait();
-            const int col0 = n_blk * BN + c * 32;
+            const int col0 = n_blk * bn + c * 32;
             if (row < p.M) {
                 __nv_bfloat16* dst = p.C + (size_t)row * p.ldc + col0;
                 const __nv_bfloat16* res = p.residual ? p.residual + (size_t)row * p.ldc + col0 : nullptr;
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
-                    if (col0 + g * 8 < p.N) {         // N is a multiple of 8
+                    if (col0 + g * 8 < col_end) {     // N is a multiple of 8
                         float x[8];
 #pragma unroll
                         for (int j = 0; j < 8; ++j) x[j] = v[g * 8 + j];
@@ -256,18 +261,19 @@ __device__ __forceinline__ void epilogue_tile(const GemmParams& p, uint32_t t_ac
             __syncwarp();
         }
     } else if (EPI == EPI_SWIGLU) {
+        const int half = bn >> 1, col_end = min(n_out, n_blk * half + half);
 #pragma unroll 1
-        for (int c = 0; c < BN / 64; ++c) {
+        for (int c = 0; c * 32 < half; ++c) {
             float g[32], u[32];
             tmem_ld32(t_acc + c * 32, g);
-            tmem_ld32(t_acc + BN / 2 + c * 32, u);
+            tmem_ld32(t_acc + half + c * 32, u);
             tmem_ld_wait();
-            const int col0 = n_blk * (BN / 2) + c * 32;
+            const int col0 = n_blk * half + c * 32;
             if (row < p.M) {
                 __nv_bfloat16* dst = p.C + (size_t)row * p.ldc + col0;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    if (col0 + q * 8 < n_out) {
+                    if (col0 + q * 8 < col_end) {
                         uint4 ov;
                         __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&ov);
 #pragma unroll

@@ -18,6 +18,13 @@ namespace jot {
 constexpr int kPairStages = 6;
 constexpr int kPairStageBytes = 2 * kBM * kBK * 2;                 // A tile + half W tile per CTA
 constexpr int kPairDynBytes = kPairStages * kPairStageBytes + 1024;
+// Tiles are walked in bands of at most this many row-block pairs where the activations are larger than kPairBandBytes: a band's rows
+// stay in L2 (126 MB, in two halves) while W streams past, where all rows in turn would come from HBM again for every column or two
+// of tiles.  11264 rows, one layer's projections at 12 / 8 / 6 / 4 / all 44 pairs a band: QKV 828 / 820 / 848 / 882 / 940 us, gate/up 1618 /
+// 1609 / 1652 / 1718 / 1821, down 851 / 847 / 870 / 904 / 960; the step 126.5 / 126.8 / 129.0 / 132.7 / 146.7 ms.  Activations that fit
+// would only read W once more per band: 4096 rows of 3584 (29 MB), gate/up 780 us in two bands, 768 in one.
+constexpr int kPairBand = 8;
+constexpr long long kPairBandBytes = 48ll << 20;
 
 // Row-block pairs and vocabulary chunks of the pair kernel's LM-head schedule.
 __host__ __device__ inline void stats_partition_pair(int R, int n_clusters, int n_vt, int* n_rb, int* n_pr, int* n_ch) {
@@ -32,10 +39,12 @@ __host__ __device__ inline void stats_partition_pair(int R, int n_clusters, int 
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
-    constexpr int BN = 256, STAGES = kPairStages;
+    constexpr int BN = 256, STAGES = kPairStages;               // BN: the widest tile, and the accumulators' stride
     constexpr uint32_t TMEM_COLS = 512;
-    constexpr uint32_t IDESC = umma_idesc_bf16(256, BN);
     constexpr int HALF_BYTES = kBM * kBK * 2;
+    const int bn = (EPI == EPI_STORE || EPI == EPI_SWIGLU) ? p.bn : BN;
+    const uint32_t idesc = umma_idesc_bf16(256, bn);
+    const uint32_t stage_tx = 2 * (uint32_t)(HALF_BYTES + bn / 2 * kBK * 2);        // bytes of both CTAs' loads per stage
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -80,9 +89,10 @@ gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, co
 
     // ---- schedule: pair tiles (two row blocks x one 256-wide column block), identical in every role ----
     const int num_m = (p.M + kBM - 1) / kBM, num_pm = (num_m + 1) / 2;
-    constexpr int BN_OUT = (EPI == EPI_SWIGLU) ? BN / 2 : BN;
+    const int bn_out = (EPI == EPI_SWIGLU) ? bn / 2 : bn;
     const int n_out = (EPI == EPI_SWIGLU) ? p.N / 2 : p.N;
-    const int num_n = (n_out + BN_OUT - 1) / BN_OUT;
+    const int num_n = (n_out + bn_out - 1) / bn_out;
+    const int band_tiles = is_stats(EPI) ? 1 : p.band * num_n;
     int total_tiles = num_pm * num_n;
     int m_blk0 = 0, n_first = 0, chunk = 0;
     bool stats_row_block_valid = false;
@@ -111,8 +121,10 @@ gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, co
         }
         const int t = cluster_id + it * n_clusters;
         if (t >= total_tiles) return false;
-        m_blk = 2 * (t % num_pm) + rank;          // row-block pairs fastest: neighbours share the W tile
-        n_blk = t / num_pm;
+        // a band of row-block pairs after the other, inside it row-block pairs fastest: neighbours share the W tile
+        const int band0 = t / band_tiles * p.band, in_band = t % band_tiles, rows_here = min(p.band, num_pm - band0);
+        m_blk = 2 * (band0 + in_band % rows_here) + rank;
+        n_blk = in_band / rows_here;
         return true;
     };
 
@@ -123,9 +135,9 @@ gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, co
         uint32_t phase = 0;
         int m_blk, n_blk;
         bool ok = true;
-        // this CTA's half of the W tile: SwiGLU pairs 128 gate rows (leader) with the matching 128 up rows
+        // this CTA's half of the W tile: SwiGLU pairs gate rows (leader) with the matching up rows
         auto w_row_of = [&](int nb) {
-            return (EPI == EPI_SWIGLU) ? (rank == 0 ? nb * kBM : p.N / 2 + nb * kBM) : nb * BN + rank * kBM;
+            return (EPI == EPI_SWIGLU) ? (rank == 0 ? nb * bn_out : p.N / 2 + nb * bn_out) : nb * bn + rank * (bn / 2);
         };
         // the first tile's first W tiles go out before the wait on the preceding kernel, its A tiles after
         int n_pre = 0;
@@ -134,7 +146,7 @@ gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, co
                 n_pre = min(STAGES, num_kb);
                 if (elected)
                     for (int i = 0; i < n_pre; ++i) {
-                        if (leader) mbar_arrive_expect_tx(&full_bar[i], 2 * kPairStageBytes);
+                        if (leader) mbar_arrive_expect_tx(&full_bar[i], stage_tx);
                         tma_load_2d_pair(smem + i * kPairStageBytes + HALF_BYTES, &tmB, mapa_u32(&full_bar[i], 0), i * kBK,
                                          w_row_of(n_blk));
                     }
@@ -158,7 +170,7 @@ gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, co
                 uint8_t* sB = sA + HALF_BYTES;
                 const uint32_t full_leader = mapa_u32(&full_bar[stage], 0);
                 if (elected) {
-                    if (leader) mbar_arrive_expect_tx(&full_bar[stage], 2 * kPairStageBytes);
+                    if (leader) mbar_arrive_expect_tx(&full_bar[stage], stage_tx);
                     tma_load_2d_pair(sA, &tmA, full_leader, kb * kBK, m_blk * kBM);
                     tma_load_2d_pair(sB, &tmB, full_leader, kb * kBK, w_row);
                 }
@@ -191,7 +203,7 @@ gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, co
                     tc_fence_after();
                     if (elected) {
 #pragma unroll
-                        for (int k = 0; k < kBK / 16; ++k) umma_bf16_pair(d_tmem, ad + 2 * k, bd + 2 * k, IDESC, accum | k);
+                        for (int k = 0; k < kBK / 16; ++k) umma_bf16_pair(d_tmem, ad + 2 * k, bd + 2 * k, idesc, accum | k);
                         umma_commit_pair(&empty_bar[stage], 0x3);     // both CTAs may refill this stage
                     }
                     __syncwarp();
@@ -222,7 +234,7 @@ gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, co
         for (int it = 0; ok && tile_at(it, m_blk, n_blk); ++it) {
             if (!mbar_wait(&acc_full[acc], acc_phase, abortp)) { ok = false; break; }
             tc_fence_after();
-            epilogue_tile<BN, EPI>(p, lane_base + acc * BN, m_blk * kBM + row_in_tile, n_blk, 0, n_out, st);
+            epilogue_tile<BN, EPI>(p, lane_base + acc * BN, m_blk * kBM + row_in_tile, n_blk, 0, n_out, st, nullptr, bn);
             tmem_ld_wait();
             tc_fence_before();
             __syncwarp();

@@ -161,9 +161,12 @@ int launch_pair_t(const GemmParams& p, const CUtensorMap& tmA, const CUtensorMap
 
 struct WeightMaps {     // one weight matrix as B operand, for both tile widths
     CUtensorMap m128, m256;
+    const void* ptr;    // and what a map of another width is made from
+    int rows, cols;
 };
 
 int make_weight_maps(const DeviceInfo* di, WeightMaps* w, const void* ptr, int rows, int cols, bool swiglu) {
+    w->ptr = ptr; w->rows = rows; w->cols = cols;
     // swiglu tiles fetch gate and up rows as two boxes of half the tile width
     JOT_TRY(make_map_2d(di, &w->m128, ptr, rows, cols, cols, swiglu ? 64 : 128));
     JOT_TRY(make_map_2d(di, &w->m256, ptr, rows, cols, cols, swiglu ? 128 : 256));
@@ -307,16 +310,28 @@ int run_slab(const DeviceInfo* di, const SlabMaps& tmX, const WeightMaps& w, int
 }
 
 // Which kernel shape moves the fewest operand bytes through an SM for this projection: waves x bytes per
-// k-block (48 KB for a 128 x 256 tile, 32 KB for a 128 x 128 tile, 32 KB per CTA of a 256 x 256 pair tile).
+// k-block (48 KB for a 128 x 256 tile, 32 KB for a 128 x 128 tile, 16 KB + bn / 2 rows of W per CTA of a 256 x bn pair tile).
+// A pair tile may be narrower than 256 columns where that fills the last wave better (a UMMA takes as long as it is wide, down to 96
+// columns); `step` is what its width is a multiple of (256: no choice).  Tiles of 256 / the width this rule finds, a step: 600 rows
+// of the LLaDA-8B shape 10.85 / 10.28 ms, 753 rows of the Dream-7B shape 10.9 / 10.1 ms (down: 130 / 107 us, in tiles of 160).
 enum { SHAPE_256 = 0, SHAPE_128 = 1, SHAPE_PAIR = 2 };
-int pick_shape(int M, int n_out, int sms, bool allow_128) {
+struct ShapePick {
+    int shape, bn;
+};
+ShapePick pick_shape(int M, int n_out, int sms, int step) {
     const long m_blks = (M + 127) / 128, n256 = (n_out + 255) / 256, n128 = (n_out + 127) / 128;
     auto waves = [](long tiles, long slots) { return (tiles + slots - 1) / slots; };
-    const long c256 = waves(m_blks * n256, sms) * 48;
-    const long c128 = allow_128 ? waves(m_blks * n128, sms) * 32 : (1L << 60);
-    const long cpair = m_blks >= 2 ? waves(((m_blks + 1) / 2) * n256, sms / 2) * 32 : (1L << 60);
-    if (c256 <= c128 && c256 <= cpair) return SHAPE_256;
-    return cpair <= c128 ? SHAPE_PAIR : SHAPE_128;
+    const long c256 = waves(m_blks * n256, sms) * 48 * 16;
+    const long c128 = waves(m_blks * n128, sms) * 32 * 16;
+    long cpair = 1L << 60;
+    int bn = 256;
+    if (m_blks >= 2)
+        for (int w = 256; w >= 128; w -= step) {
+            const long c = waves((m_blks + 1) / 2 * ((n_out + w - 1) / w), sms / 2) * (16 * 16 + w);
+            if (c < cpair) { cpair = c; bn = w; }
+        }
+    if (c256 <= c128 && c256 <= cpair) return {SHAPE_256, 256};
+    return cpair <= c128 ? ShapePick{SHAPE_PAIR, bn} : ShapePick{SHAPE_128, 128};
 }
 
 // Split-K factor for a plain projection: when 256-wide tiles leave most SMs idle, cut K into up to 4
@@ -367,16 +382,22 @@ int run_gemm(const DeviceInfo* di, const CUtensorMap& tmA, const WeightMaps& w, 
     // for SwiGLU a "256-wide" tile holds 128 gate + 128 up columns, i.e. 128 output columns
     const int n_out = (epi == EPI_SWIGLU) ? p.N / 2 : p.N;
     const int n_eff = (epi == EPI_SWIGLU) ? 2 * n_out : n_out;
-    const int shape = pick_shape(p.M, n_eff, di->sms, true);
-    if (shape == SHAPE_PAIR) {
-        const long tiles = (long)(((p.M + 127) / 128 + 1) / 2) * ((n_eff + 255) / 256);
+    const ShapePick pick = pick_shape(p.M, n_eff, di->sms, epi == EPI_QKV ? 256 : (epi == EPI_SWIGLU ? 32 : 16));
+    if (pick.shape == SHAPE_PAIR) {
+        const long pair_rows = ((p.M + 127) / 128 + 1) / 2, tiles = pair_rows * ((n_eff + pick.bn - 1) / pick.bn);
         const int grid = (int)(2 * tiles < di->sms ? 2 * tiles : di->sms);
-        // each CTA of a pair fetches 128 rows of W: the 128-row box of the plain maps, the 128-row box of SwiGLU's
-        if (epi == EPI_STORE) return launch_pair_t<EPI_STORE>(p, tmA, w.m128, grid, st);
-        if (epi == EPI_QKV) return launch_pair_t<EPI_QKV>(p, tmA, w.m128, grid, st);
-        return launch_pair_t<EPI_SWIGLU>(p, tmA, w.m256, grid, st);
+        p.bn = pick.bn;
+        const long bands = 2ll * p.M * p.K <= kPairBandBytes ? 1 : (pair_rows + kPairBand - 1) / kPairBand;
+        p.band = (int)((pair_rows + bands - 1) / bands);
+        // each CTA of a pair fetches half of the tile's rows of W (SwiGLU: one its gate rows, the other its up rows)
+        CUtensorMap narrow;
+        if (pick.bn < 256) JOT_TRY(make_map_2d(di, &narrow, w.ptr, w.rows, w.cols, w.cols, (uint32_t)pick.bn / 2));
+        const CUtensorMap& tmB = pick.bn < 256 ? narrow : (epi == EPI_SWIGLU ? w.m256 : w.m128);
+        if (epi == EPI_STORE) return launch_pair_t<EPI_STORE>(p, tmA, tmB, grid, st);
+        if (epi == EPI_QKV) return launch_pair_t<EPI_QKV>(p, tmA, tmB, grid, st);
+        return launch_pair_t<EPI_SWIGLU>(p, tmA, tmB, grid, st);
     }
-    const int bn = shape == SHAPE_128 ? 128 : 256;
+    const int bn = pick.bn;
     const int bn_out = (epi == EPI_SWIGLU) ? bn / 2 : bn;
     long tiles = (long)((p.M + 127) / 128) * ((n_out + bn_out - 1) / bn_out);
     int grid = (int)(tiles < di->sms ? tiles : di->sms);

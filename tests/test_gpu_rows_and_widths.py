@@ -42,3 +42,10 @@ def geometry(d, heads, hd, ff, layers=2):
 @pytest.mark.parametrize("d,B,L", [(64, 1, 20), (4096, 1, 20), (4160, 1, 20), (8256, 1, 20), (320, 9, 133)])     # ... and more rows than CTAs
 def test_norm_widths(jot, d, B, L):
     check_step(jot, geometry(d, 2, 64, 128, layers=1), B, L)
+
+
+# pair tiles narrower than 256 columns: halves of 112 and of 64 gate columns, O and down in tiles of 240 and less; the last tile and
+# the last row block ragged; more row blocks than a band has
+@pytest.mark.parametrize("d,ff,B,L", [(256, 1984, 8, 125), (256, 1024, 8, 125), (512, 3968, 4, 130), (4096, 512, 8, 125), (256, 512, 18, 131)])
+def test_pair_tile_widths(jot, d, ff, B, L):
+    check_step(jot, geometry(d, d // 64, 64, ff, layers=1), B, L)
