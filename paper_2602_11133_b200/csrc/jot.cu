@@ -20,6 +20,7 @@
 #include "gemm.cuh"
 #include "gemm2.cuh"
 #include "gemm_slab.cuh"
+#include "gemm_stream.cuh"
 #include "glue.cuh"
 
 using namespace jot;
@@ -246,6 +247,29 @@ int launch_slab_gateup2(GemmParams p, const CUtensorMap& tmW, const SlabMaps& tm
     return launch_check();
 }
 
+// ---------------------------------------------------------------- stream kernels (small canvases)
+template <typename... KArgs, typename... Args>
+int launch_stream(void (*kernel)(KArgs...), bool* attr_set, int ctas, int smem, cudaStream_t st, Args&&... args) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (!attr_set[dev & 63]) {
+        JOT_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStreamSmem));
+        attr_set[dev & 63] = true;
+    }
+    launch_k(kernel, dim3((unsigned)ctas), dim3(kStreamThreads), (size_t)smem, st, args...);
+    return launch_check();
+}
+
+// Gate/up + SwiGLU of a small canvas; tmX: boxes of all tokens.
+int run_stream_gateup(const DeviceInfo* di, const CUtensorMap& tmX, const WeightMaps& w, const GemmParams& p, cudaStream_t st) {
+    static thread_local bool attr_set[64] = {};
+    const int n_out = p.N / 2, rows = stream_gateup_rows(n_out, di->sms);
+    CUtensorMap tmW;
+    JOT_TRY(make_map_2d(di, &tmW, w.ptr, w.rows, w.cols, w.cols, (uint32_t)rows));
+    return launch_stream(gemm_stream_gateup_kernel, attr_set, std::min(di->sms, (n_out + rows - 1) / rows),
+                         stream_geom(p.M, 2 * rows, (p.M + 15) / 16 * 16).smem_bytes, st, p, rows, tmW, tmX);
+}
+
 // How many clusters of `split` pairs the device runs side by side (1 CTA per SM: the kernel takes all shared memory).
 int slab_cluster_capacity(int sms, int split) {
     static thread_local int cap[64][5] = {};
@@ -354,9 +378,43 @@ struct NormAfter {
     bool done;
 };
 
+// The K ranges' sums, the residual and the norm: the tail of a split projection.
+int launch_reduce_norm(const float* scratch, int split, const GemmParams& p, NormAfter* norm, cudaStream_t st) {
+    int threads = (p.N / 8 + 31) / 32 * 32;      // one 8-element vector per thread up to 512 threads
+    threads = threads > 512 ? 512 : (threads < 64 ? 64 : threads);
+    launch_k(p.N / 8 <= threads ? splitk_reduce_norm_kernel<1> : splitk_reduce_norm_kernel<2>, dim3(p.M), dim3(threads), 0, st, scratch, split,
+             p.residual, p.C, p.M, p.N, norm->gain, norm->out, norm->eps);
+    norm->done = true;
+    return launch_check();
+}
+
+// A projection with residual whose output is normalised next, as a stream of weights in K ranges over the CTA pairs.  Needs
+// `scratch` for the ranges' sums.
+bool stream_split(const DeviceInfo* di, const GemmParams& p, size_t scratch_bytes, const NormAfter* norm, int* split) {
+    if (!norm || p.ldc != p.N || p.N / 8 > 1024 || p.M > kStreamMaxTokens) return false;
+    const int slabs = (p.N + 255) / 256, num_kb = (p.K + kBK - 1) / kBK;
+    int s = di->sms / 2 / slabs;
+    s = s > 4 ? 4 : s;
+    while (s > 1 && (num_kb / s < 4 || (size_t)s * p.M * p.N * 4 > scratch_bytes)) --s;
+    *split = s;
+    return s >= 1 && (size_t)s * p.M * p.N * 4 <= scratch_bytes;
+}
+int run_stream_partial(const CUtensorMap& tmX, const WeightMaps& w, GemmParams p, int split, float* scratch, NormAfter* norm, cudaStream_t st) {
+    static thread_local bool attr_set[64] = {};
+    p.split_k = split;
+    p.partial = scratch;
+    JOT_TRY(launch_stream(gemm_stream_partial_kernel, attr_set, 2 * split * ((p.N + 255) / 256), stream_geom(p.M, 128, (p.M + 15) / 16 * 8).smem_bytes, st,
+                          p, w.m128, tmX));
+    return launch_reduce_norm(scratch, split, p, norm, st);
+}
+
 int run_gemm(const DeviceInfo* di, const CUtensorMap& tmA, const WeightMaps& w, int epi, GemmParams p, cudaStream_t st,
              float* scratch = nullptr, size_t scratch_bytes = 0, NormAfter* norm = nullptr,
-             const SlabMaps* tmX_slab = nullptr) {
+             const SlabMaps* tmX_slab = nullptr, const CUtensorMap* tmX_stream = nullptr) {
+    int split_s = 0;
+    if (tmX_stream && epi == EPI_STORE && stream_split(di, p, scratch_bytes, norm, &split_s))
+        return run_stream_partial(*tmX_stream, w, p, split_s, scratch, norm, st);
+    if (tmX_stream && epi == EPI_SWIGLU) return run_stream_gateup(di, *tmX_stream, w, p, st);
     // small canvases: weight rows as the MMA's M side, every token in tensor memory (gemm_slab.cuh)
     if (tmX_slab && p.M <= kSlabMaxTokens) return run_slab(di, *tmX_slab, w, epi, p, st);      // callers decide when
     if (epi == EPI_STORE && scratch) {
@@ -366,14 +424,7 @@ int run_gemm(const DeviceInfo* di, const CUtensorMap& tmA, const WeightMaps& w, 
             p.partial = scratch;
             const long items = (long)((p.M + 127) / 128) * ((p.N + 255) / 256) * split;
             JOT_TRY((launch_gemm_t<256, EPI_PARTIAL>(p, tmA, w.m256, (int)items, st)));
-            if (norm && p.ldc == p.N && p.N / 8 <= 1024) {
-                int threads = (p.N / 8 + 31) / 32 * 32;      // one 8-element vector per thread up to 512 threads
-                threads = threads > 512 ? 512 : (threads < 64 ? 64 : threads);
-                launch_k(p.N / 8 <= threads ? splitk_reduce_norm_kernel<1> : splitk_reduce_norm_kernel<2>, dim3(p.M), dim3(threads), 0,
-                         st, scratch, split, p.residual, p.C, p.M, p.N, norm->gain, norm->out, norm->eps);
-                norm->done = true;
-                return launch_check();
-            }
+            if (norm && p.ldc == p.N && p.N / 8 <= 1024) return launch_reduce_norm(scratch, split, p, norm, st);
             const size_t n8 = (size_t)p.M * p.N / 8;
             launch_k(splitk_reduce_kernel, dim3((unsigned)((n8 + 255) / 256)), dim3(256), 0, st, scratch, split, p.residual, p.C, p.M, p.N);
             return launch_check();
@@ -474,7 +525,8 @@ struct jot_model {
     // A-operand maps of the projections for a pass over M rows (rows past M read as zero without memory
     // traffic): one set for the whole canvas, one for the rows of a block
     // (x*: the same buffers as the token operand of the slab kernel, boxes of half an accumulator's tokens)
-    struct ActMaps { int M = -1; bool slab = false, slab_gate_up = false; CUtensorMap a, attn, act; SlabMaps xa, xattn, xact; };
+    struct ActMaps { int M = -1; bool slab = false, slab_gate_up = false, stream = false; CUtensorMap a, attn, act;
+                     SlabMaps xa, xattn, xact; CUtensorMap sa, sattn, sact; };
     ActMaps maps_full, maps_span;
     // block-wise KV cache (caller's memory, optional): per layer the rotated Q/K rows and V^T of the whole canvas
     uint8_t* kv_base = nullptr;
@@ -603,9 +655,14 @@ int encode_act_maps(jot_model* m, jot_model::ActMaps* am, int M) {
     JOT_TRY(make_map_2d(m->di, &am->attn, m->attn, M, c.n_q_heads * c.head_dim, c.n_q_heads * c.head_dim, 128));
     JOT_TRY(make_map_2d(m->di, &am->act, m->act, M, c.d_ff, c.d_ff, 128));
     am->slab = M <= kSlabPreferTokens;
-    am->slab_gate_up = (M > 128 && M <= kSlabGateUpTokens) ||
-                       ((2 * c.d_ff) % 256 == 0 &&
-                        slab2_plan(M, 2 * c.d_ff / 256, slab_cluster_capacity(m->di->sms, 1)).ok);
+    am->stream = M <= kStreamMaxTokens;
+    am->slab_gate_up = (2 * c.d_ff) % 256 == 0 && slab2_plan(M, 2 * c.d_ff / 256, slab_cluster_capacity(m->di->sms, 1)).ok;
+    if (am->stream) {
+        const uint32_t tokens = (uint32_t)((M + 15) / 16 * 16);
+        JOT_TRY(make_map_2d(m->di, &am->sa, m->a, M, c.d_model, c.d_model, tokens));
+        JOT_TRY(make_map_2d(m->di, &am->sattn, m->attn, M, c.n_q_heads * c.head_dim, c.n_q_heads * c.head_dim, tokens / 2));
+        JOT_TRY(make_map_2d(m->di, &am->sact, m->act, M, c.d_ff, c.d_ff, tokens / 2));
+    }
     if (am->slab || am->slab_gate_up) {
         JOT_TRY(make_slab_maps(m->di, &am->xa, m->a, M, c.d_model, c.d_model));
         JOT_TRY(make_slab_maps(m->di, &am->xattn, m->attn, M, c.n_q_heads * c.head_dim, c.n_q_heads * c.head_dim));
@@ -701,7 +758,7 @@ int forward_body(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStream
             ProfScope ps(m, JOT_PROF_GEMM_O, st);
             NormAfter na{m->mlp_norm[l], m->a, c.rms_eps, false};
             JOT_TRY(run_gemm(m->di, am.attn, m->wo[l], EPI_STORE, p, st, m->splitk, kSplitKBytes, &na,
-                             am.slab ? &am.xattn : nullptr));
+                             am.slab ? &am.xattn : nullptr, am.stream ? &am.sattn : nullptr));
             norm_ready = na.done;
         }
         if (!norm_ready) {
@@ -712,10 +769,8 @@ int forward_body(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStream
         p.M = M; p.N = 2 * c.d_ff; p.K = d; p.C = m->act; p.ldc = c.d_ff; p.status = status;
         {
             ProfScope ps(m, JOT_PROF_GEMM_GATE_UP, st);
-            // (up to 128 rows the token-major tiles stream the gate/up weights faster than the slab kernel's two
-            // launches do: measured 39-43 us against 42-47)
             JOT_TRY(run_gemm(m->di, am.a, m->wgu[l], EPI_SWIGLU, p, st, nullptr, 0, nullptr,
-                             am.slab_gate_up ? &am.xa : nullptr));
+                             am.slab_gate_up ? &am.xa : nullptr, am.stream ? &am.sa : nullptr));
         }
         p = GemmParams{};
         p.M = M; p.N = d; p.K = c.d_ff; p.C = m->h; p.residual = m->h; p.ldc = d; p.status = status;
@@ -723,7 +778,7 @@ int forward_body(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStream
             ProfScope ps(m, JOT_PROF_GEMM_DOWN, st);
             NormAfter na{l + 1 < c.n_layers ? m->attn_norm[l + 1] : nullptr, m->a, c.rms_eps, false};
             JOT_TRY(run_gemm(m->di, am.act, m->wdown[l], EPI_STORE, p, st, m->splitk, kSplitKBytes,
-                             na.gain ? &na : nullptr, am.slab ? &am.xact : nullptr));
+                             na.gain ? &na : nullptr, am.slab ? &am.xact : nullptr, am.stream ? &am.sact : nullptr));
             norm_ready = na.done;
         }
     }

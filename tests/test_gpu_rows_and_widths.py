@@ -49,3 +49,24 @@ def test_norm_widths(jot, d, B, L):
 @pytest.mark.parametrize("d,ff,B,L", [(256, 1984, 8, 125), (256, 1024, 8, 125), (512, 3968, 4, 130), (4096, 512, 8, 125), (256, 512, 18, 131)])
 def test_pair_tile_widths(jot, d, ff, B, L):
     check_step(jot, geometry(d, d // 64, 64, ff, layers=1), B, L)
+
+
+# gate/up as two units per pair: a K of fewer blocks than stages, of as many, and more
+@pytest.mark.parametrize("d", [64, 128, 192, 320, 576])
+@pytest.mark.parametrize("B,L", [(1, 353), (1, 384)])
+def test_two_unit_gate_up(jot, d, B, L):
+    check_step(jot, geometry(d, d // 64, 64, 12288, layers=1), B, L)
+
+
+# gate/up dealt over the SMs eight features at a time: 704 (a CTA of 8 each), 9600 (72, the last one ragged), 18944 (128 each), 19200 (two
+# units a CTA)
+@pytest.mark.parametrize("ff", [704, 9600, 18944, 19200])
+@pytest.mark.parametrize("B,L", [(1, 1), (1, 16), (1, 17), (3, 11), (1, 128), (1, 144), (5, 29), (1, 255), (1, 256)])
+def test_small_canvases(jot, ff, B, L):
+    check_step(jot, geometry(256, 4, 64, ff), B, L)
+
+
+# wide layers of few rows: four K ranges of O and down, a ragged last slab of 64 of 256 features
+@pytest.mark.parametrize("B,L", [(1, 33), (1, 133), (2, 120)])
+def test_small_canvases_of_long_sums(jot, B, L):
+    check_step(jot, geometry(1344, 24, 128, 3200, layers=1), B, L)
