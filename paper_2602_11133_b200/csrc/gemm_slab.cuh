@@ -23,7 +23,6 @@
 // of four warps (128 features) turns its 32-token chunk around through a 16 KB fp32 buffer in shared memory
 // (the pipeline's stages, free by then) and leaves with 16-byte stores:
 //     SLAB_STORE   bf16(acc [+ residual])
-//     SLAB_SWIGLU  a CTA's 128 rows are 64 gate rows and the matching 64 up rows: bf16(silu(g) * u)
 //     SLAB_QKV     bf16(acc), rotary embedding on Q and K heads (the partner feature sits 64 lanes away, the
 //                  buffer brings them together), V heads written transposed straight from the registers
 //                  (a thread's 32 tokens are 64 contiguous bytes of V^T)
@@ -38,12 +37,8 @@ constexpr int kSlabMaxTokens = 512;        // two accumulators of 256 fp32 colum
 #define JOT_SLAB_PREFER_TOKENS 256
 #endif
 constexpr int kSlabPreferTokens = JOT_SLAB_PREFER_TOKENS;   // measured: up to here this kernel beats the token-major tiles
-#ifndef JOT_SLAB_GATEUP_TOKENS
-#define JOT_SLAB_GATEUP_TOKENS JOT_SLAB_PREFER_TOKENS
-#endif
-constexpr int kSlabGateUpTokens = JOT_SLAB_GATEUP_TOKENS;   // the same switch for the gate/up projection alone
 constexpr int kSlabMaxSmem = 226 * 1024;   // dynamic part; the static barriers take the rest of the 227 KB
-enum { SLAB_STORE = 0, SLAB_SWIGLU = 1, SLAB_QKV = 2 };
+enum { SLAB_STORE = 0, SLAB_SWIGLU = 1, SLAB_QKV = 2 };      // (SLAB_SWIGLU: the two-unit kernel below)
 
 // How a canvas of M rows maps onto accumulators, and what a launch needs in shared memory.  The tensor pipe
 // spends as long on a UMMA of 192 columns as on one of 256 (measured), so the first accumulator always
@@ -144,7 +139,7 @@ gemm_slab_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmW, co
     // tiles BEFORE that wait and the pipeline's fill latency overlaps the predecessor's tail.
 
     // first weight row of this CTA's tile(s)
-    const int f0 = (EPI == SLAB_SWIGLU) ? (2 * slab + pr) * 64 : (2 * slab + pr) * 128;
+    const int f0 = (2 * slab + pr) * 128;
 
     if (warp == 0) {
         // ================= TMA producer (the whole warp runs the loop, one lane issues) =================
@@ -153,13 +148,7 @@ gemm_slab_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmW, co
         auto load_w = [&](int stage, int kb, uint32_t full_leader) {
             uint8_t* sW = smem + stage * g.stage_bytes;
             if (leader) mbar_arrive_expect_tx(&full_bar[stage], 2 * g.stage_bytes);
-            if (EPI == SLAB_SWIGLU) {
-                // 64 gate rows, then the 64 up rows of the same output features
-                tma_load_2d_pair_hint(sW, &tmW, full_leader, kb * kBK, f0, once);
-                tma_load_2d_pair_hint(sW + 64 * 128, &tmW, full_leader, kb * kBK, p.N / 2 + f0, once);
-            } else {
-                tma_load_2d_pair_hint(sW, &tmW, full_leader, kb * kBK, f0, once);
-            }
+            tma_load_2d_pair_hint(sW, &tmW, full_leader, kb * kBK, f0, once);
         };
         auto load_x = [&](int stage, int kb, uint32_t full_leader) {
             // this CTA's half of every accumulator's token tile
@@ -441,27 +430,6 @@ gemm_slab_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmW, co
                         *reinterpret_cast<uint4*>(p.C + (size_t)t * p.ldc + oc) = ov;
                     }
                     if (p.residual && more) load_residual(c + 2);
-                } else if (EPI == SLAB_SWIGLU) {
-                    const int n_out = p.N / 2;
-#pragma unroll 1
-                    for (int item = tid_g; item < 32 * 8; item += 128) {
-                        const int tok = item >> 3, gq = item & 7, t = t0 + tok, oc = f0 + gq * 8;
-                        if (t >= p.M || oc >= n_out) continue;
-                        const float* gp = sb + tok * 128 + gq * 8;
-                        const float4 g0 = *reinterpret_cast<const float4*>(gp), g1 = *reinterpret_cast<const float4*>(gp + 4);
-                        const float4 u0 = *reinterpret_cast<const float4*>(gp + 64), u1 = *reinterpret_cast<const float4*>(gp + 68);
-                        const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-                        const float uu[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-                        uint4 ov;
-                        __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&ov);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const float a0 = silu_mul(gg[2 * j], uu[2 * j]);
-                            const float a1 = silu_mul(gg[2 * j + 1], uu[2 * j + 1]);
-                            o2[j] = __floats2bfloat162_rn(a0, a1);
-                        }
-                        *reinterpret_cast<uint4*>(p.C + (size_t)t * p.ldc + oc) = ov;
-                    }
                 } else {
                     // Q and K heads: pairs (j, j + hd/2) of one head, 8 pairs per item
                     const int hd = p.hd, half = hd >> 1;

@@ -311,21 +311,18 @@ int slab_pick_split(int M, int n_slabs, int num_kb, int sms) {
 }
 
 int run_slab(const DeviceInfo* di, const SlabMaps& tmX, const WeightMaps& w, int epi, const GemmParams& p, cudaStream_t st) {
-    const int n_out = (epi == EPI_SWIGLU) ? p.N / 2 : p.N;
-    const int per_slab = (epi == EPI_SWIGLU) ? 128 : 256;                 // output features per CTA pair
-    const int n_slabs = (n_out + per_slab - 1) / per_slab;
+    const int n_slabs = (p.N + 255) / 256;                                // 256 rows of W per CTA pair
     const int num_kb = (p.K + kBK - 1) / kBK;
+    const int cap1 = slab_cluster_capacity(di->sms, 1);
+    if (epi == EPI_SWIGLU) {                                              // callers ask the plan before they come here
+        const Slab2Plan plan = slab2_plan(p.M, n_slabs, cap1);
+        return plan.ok ? launch_slab_gateup2(p, w.m128, tmX, plan, st) : JOT_ERR_SHAPE;
+    }
     auto go = [&](int slab0, int n, int split) -> int {
         if (n <= 0) return JOT_OK;
         if (epi == EPI_STORE) return launch_slab_t<SLAB_STORE>(p, w.m128, tmX, slab0, n, split, st);
-        if (epi == EPI_QKV) return launch_slab_t<SLAB_QKV>(p, w.m128, tmX, slab0, n, split, st);
-        return launch_slab_t<SLAB_SWIGLU>(p, w.m128, tmX, slab0, n, split, st);
+        return launch_slab_t<SLAB_QKV>(p, w.m128, tmX, slab0, n, split, st);
     };
-    const int cap1 = slab_cluster_capacity(di->sms, 1);
-    if (epi == EPI_SWIGLU && p.N % 256 == 0) {
-        const Slab2Plan plan = slab2_plan(p.M, n_slabs, cap1);
-        if (plan.ok) return launch_slab_gateup2(p, w.m128, tmX, plan, st);
-    }
     // whole waves of unsplit slabs first; what is left over (or a projection with few slabs) is cut along K so
     // that it still fills the machine
     const int full = n_slabs / cap1 * cap1, rest = n_slabs - full;
