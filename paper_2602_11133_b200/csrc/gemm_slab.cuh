@@ -40,9 +40,8 @@ constexpr int kSlabPreferTokens = JOT_SLAB_PREFER_TOKENS;   // measured: up to h
 constexpr int kSlabMaxSmem = 226 * 1024;   // dynamic part; the static barriers take the rest of the 227 KB
 enum { SLAB_STORE = 0, SLAB_SWIGLU = 1, SLAB_QKV = 2 };      // (SLAB_SWIGLU: the two-unit kernel below)
 
-// How a canvas of M rows maps onto accumulators, and what a launch needs in shared memory.  The tensor pipe
-// spends as long on a UMMA of 192 columns as on one of 256 (measured), so the first accumulator always
-// takes 256 tokens when there are more than that and the second one the rest.
+// How a canvas of M rows maps onto accumulators, and what a launch needs in shared memory: the first accumulator takes 256 tokens
+// when there are more than that and the second one the rest.
 struct SlabGeom {
     int n_acc;          // accumulators (UMMAs per k-step)
     int n0, n1;         // token columns of the two accumulators: multiples of 32, at most 256 (n1 = 0: one only)
