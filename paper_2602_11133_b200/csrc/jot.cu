@@ -332,9 +332,11 @@ int run_slab(const DeviceInfo* di, const SlabMaps& tmX, const WeightMaps& w, int
 
 // Which kernel shape moves the fewest operand bytes through an SM for this projection: waves x bytes per
 // k-block (48 KB for a 128 x 256 tile, 32 KB for a 128 x 128 tile, 16 KB + bn / 2 rows of W per CTA of a 256 x bn pair tile).
-// A pair tile may be narrower than 256 columns where that fills the last wave better (a UMMA takes as long as it is wide, down to 96
-// columns); `step` is what its width is a multiple of (256: no choice).  Tiles of 256 / the width this rule finds, a step: 600 rows
-// of the LLaDA-8B shape 10.85 / 10.28 ms, 753 rows of the Dream-7B shape 10.9 / 10.1 ms (down: 130 / 107 us, in tiles of 160).
+// Among pair tiles one may then be narrower than 256 columns where that fills the last wave better (a UMMA takes as long as it is wide,
+// down to 96 columns); `step` is what its width is a multiple of (256: no choice).  Tiles of 256 / the width this rule finds, a step: 600
+// rows of the LLaDA-8B shape 10.85 / 10.28 ms, 753 rows of the Dream-7B shape 10.9 / 10.1 ms (down: 130 / 107 us, in tiles of 160).
+// A narrower tile is no reason to take pairs in place of the other shapes: 257 to 352 rows of the LLaDA-8B shape, gate/up in one-CTA
+// tiles 58-68 us, in three waves of pair tiles of 224 columns 70-83.
 enum { SHAPE_256 = 0, SHAPE_128 = 1, SHAPE_PAIR = 2 };
 struct ShapePick {
     int shape, bn;
@@ -344,15 +346,14 @@ ShapePick pick_shape(int M, int n_out, int sms, int step) {
     auto waves = [](long tiles, long slots) { return (tiles + slots - 1) / slots; };
     const long c256 = waves(m_blks * n256, sms) * 48 * 16;
     const long c128 = waves(m_blks * n128, sms) * 32 * 16;
-    long cpair = 1L << 60;
-    int bn = 256;
-    if (m_blks >= 2)
-        for (int w = 256; w >= 128; w -= step) {
-            const long c = waves((m_blks + 1) / 2 * ((n_out + w - 1) / w), sms / 2) * (16 * 16 + w);
-            if (c < cpair) { cpair = c; bn = w; }
-        }
+    auto pair_cost = [&](int w) { return waves((m_blks + 1) / 2 * ((n_out + w - 1) / w), sms / 2) * (16 * 16 + w); };
+    long cpair = m_blks >= 2 ? pair_cost(256) : (1L << 60);
     if (c256 <= c128 && c256 <= cpair) return {SHAPE_256, 256};
-    return cpair <= c128 ? ShapePick{SHAPE_PAIR, bn} : ShapePick{SHAPE_128, 128};
+    if (c128 < cpair) return {SHAPE_128, 128};
+    int bn = 256;
+    for (int w = 256 - step; w >= 128; w -= step)
+        if (pair_cost(w) < cpair) { cpair = pair_cost(w); bn = w; }
+    return {SHAPE_PAIR, bn};
 }
 
 // Split-K factor for a plain projection: when 256-wide tiles leave most SMs idle, cut K into up to 4

@@ -70,3 +70,27 @@ def test_small_canvases(jot, ff, B, L):
 @pytest.mark.parametrize("B,L", [(1, 33), (1, 133), (2, 120)])
 def test_small_canvases_of_long_sums(jot, B, L):
     check_step(jot, geometry(1344, 24, 128, 3200, layers=1), B, L)
+
+
+# gate/up of the LLaDA-8B widths: 257 to 352 rows are less work than 384 and take no longer (pair tiles of 224 columns took 1.07 times as long)
+def test_fewer_rows_take_no_longer(jot):
+    g = geometry(4096, 32, 128, 12288, layers=1)
+    weights = inputs.model_weights(g, seed=0, device="cuda")
+
+    def gate_up(L):
+        model = jot.Model(g, weights, 1, L)
+        tokens = torch.full((1, L), 5, dtype=torch.int32, device="cuda")
+        best = float("inf")
+        for _ in range(8):
+            model.profile(True)
+            for _ in range(10):
+                model.denoise_step(tokens, 0, 0)
+            ms, spans = model.profile_read()["gemm_gate_up"]
+            best = min(best, ms / spans)
+            model.profile(False)
+        model.close()
+        return best
+
+    full = gate_up(384)
+    for rows in (257, 300, 352):
+        assert gate_up(rows) < full, rows
