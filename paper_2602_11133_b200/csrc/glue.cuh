@@ -132,14 +132,14 @@ rmsnorm_kernel(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restr
     }
 }
 
-// Split-K tail fused with the next RMSNorm: one CTA per row, one (at most two) 8-element vectors per thread,
+// Split-K tail fused with the next RMSNorm: one CTA per row, one (at most four) 8-element vectors per thread,
 // every load of a thread issued before the first use so that a row costs one round trip to L2.
 //   h[row, :]   = bf16( sum over K ranges of partial + residual )          (the projection's output)
 //   out[row, :] = bf16( h * rsqrt(mean(h^2) + eps) * gain )                (h as rounded, like rmsnorm_kernel)
-// N multiple of 8, N/8 <= MAXV * blockDim.x (at most 512 threads), split <= 4.  One vector per thread is an instance of its
-// own: at 62 registers instead of 114 two rows share an SM (384 rows of 4096 columns, three ranges: 9.8 -> 7.6 us).
+// N multiple of 8, N/8 <= MAXV * blockDim.x (at most 512 threads; 256 with four vectors), split <= 4.  One vector per thread is an
+// instance of its own: at 62 registers instead of 114 two rows share an SM (384 rows of 4096 columns, three ranges: 9.8 -> 7.6 us).
 template <int MAXV>
-__global__ void __launch_bounds__(512, MAXV == 1 ? 2 : 1) splitk_reduce_norm_kernel(const float* __restrict__ partial, int split,
+__global__ void __launch_bounds__(MAXV <= 2 ? 512 : 256, MAXV == 1 ? 2 : 1) splitk_reduce_norm_kernel(const float* __restrict__ partial, int split,
                                                                   const __nv_bfloat16* residual, __nv_bfloat16* C, int M,
                                                                   int N, const __nv_bfloat16* __restrict__ gain,
                                                                   __nv_bfloat16* __restrict__ out, float eps) {

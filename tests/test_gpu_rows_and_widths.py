@@ -72,6 +72,51 @@ def test_small_canvases_of_long_sums(jot, B, L):
     check_step(jot, geometry(1344, 24, 128, 3200, layers=1), B, L)
 
 
+def statistics(jot, g, weights, tokens, lo):
+    model = jot.Model(g, weights, *tokens.shape)
+    st = model.denoise_step(tokens, lo, tokens.shape[1])
+    model.close()
+    return [t[:, lo:] for t in (st.top1, st.top2, st.sumexp, st.argmax)]
+
+
+def masked_canvas(g, B, L, n_masked):
+    tokens = inputs.token_ids(3, "canvas", B * L, g.vocab, g.mask_id, device="cuda").view(B, L)
+    tokens[:, L - n_masked:] = g.mask_id
+    return tokens
+
+
+# down adds the same K ranges in the same order with a norm behind it (streams) and as the last layer's (slabs): a second layer that
+# adds nothing changes no bit
+@pytest.mark.parametrize("d,heads,hd,ff", [(256, 4, 64, 704), (3584, 28, 128, 2048), (4096, 32, 128, 3072), (4672, 4, 64, 2048), (8192, 4, 64, 1088)])
+@pytest.mark.parametrize("L", [20, 133, 256])
+def test_same_bits_with_a_norm_behind_and_without(jot, d, heads, hd, ff, L):
+    g = geometry(d, heads, hd, ff)
+    weights = inputs.model_weights(g, seed=0, device="cuda")
+    tokens = masked_canvas(g, 1, L, 16)
+    first, second = weights["layers"]
+    nothing = dict(second, wo=torch.zeros_like(second["wo"]), w_down=torch.zeros_like(second["w_down"]))
+    one = statistics(jot, g, dict(weights, layers=[first]), tokens, L - 16)
+    two = statistics(jot, g, dict(weights, layers=[first, nothing]), tokens, L - 16)
+    for a, b in zip(one, two):
+        assert torch.equal(a, b)
+
+
+# the norm in the tail of a split projection adds a row's squares in the order of the norm on its own: a sequence gets the same bits
+# alone and in a batch, where no projection is split (O and down have one K range that is not zero, so that their sums are the same)
+@pytest.mark.parametrize("d,heads,hd", [(3584, 28, 128), (4096, 32, 128), (5120, 32, 128)])
+def test_same_bits_of_both_norms(jot, d, heads, hd):
+    g = geometry(d, heads, hd, 4096)
+    weights = inputs.model_weights(g, seed=0, device="cuda")
+    for layer in weights["layers"]:
+        layer["wo"][:, heads * hd // 256 * 64:] = 0
+        layer["w_down"][:, g.d_ff // 4:] = 0
+    tokens = masked_canvas(g, 9, 100, 8)
+    batch = statistics(jot, g, weights, tokens, 92)
+    for b in (0, 8):
+        for x, y in zip(statistics(jot, g, weights, tokens[b:b + 1].contiguous(), 92), batch):
+            assert torch.equal(x[0], y[b])
+
+
 # gate/up of the LLaDA-8B widths: 257 to 352 rows are less work than 384 and take no longer (pair tiles of 224 columns took 1.07 times as long)
 def test_fewer_rows_take_no_longer(jot):
     g = geometry(4096, 32, 128, 12288, layers=1)
