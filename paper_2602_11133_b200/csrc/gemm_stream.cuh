@@ -209,8 +209,7 @@ gemm_stream_partial_kernel(const GemmParams p, const __grid_constant__ CUtensorM
 // tensor memory has room).  Gate and up rows are two UMMAs of M = 128 into two accumulators: feature f's gate and up products sit in the
 // same TMEM lane, so SwiGLU needs no exchange and a warp writes 32 consecutive outputs of a token.  Against 96 token-major tiles (32
 // rows, LLaDA-8B shape) 44.6 -> 43.0 us between events, and the step 3575 -> 3425; against two waves of slabs (133 rows, Dream-7B shape)
-// 62.5 -> 55.5, 3810 -> 3645; 256 rows of it 75 -> 68.  The LLaDA-8B shape at 128 and 200 rows takes 1.5 and 0.7 % longer a step than with
-// the tiles and slabs, one rule for all being worth that.
+// 62.5 -> 55.5, 3810 -> 3645.  Which passes come here: stream_gateup_pays (jot.cu).
 __host__ __device__ inline int stream_gateup_rows(int n_out, int ctas) {
     const int groups = (n_out + 7) / 8, waves = (groups + 16 * ctas - 1) / (16 * ctas);
     return 8 * ((groups + waves * ctas - 1) / (waves * ctas));

@@ -340,6 +340,7 @@ int run_slab(const DeviceInfo* di, const SlabMaps& tmX, const WeightMaps& w, int
 enum { SHAPE_256 = 0, SHAPE_128 = 1, SHAPE_PAIR = 2 };
 struct ShapePick {
     int shape, bn;
+    long cost;          // waves x bytes per k-block, in units of 64 bytes
 };
 ShapePick pick_shape(int M, int n_out, int sms, int step) {
     const long m_blks = (M + 127) / 128, n256 = (n_out + 255) / 256, n128 = (n_out + 127) / 128;
@@ -348,12 +349,30 @@ ShapePick pick_shape(int M, int n_out, int sms, int step) {
     const long c128 = waves(m_blks * n128, sms) * 32 * 16;
     auto pair_cost = [&](int w) { return waves((m_blks + 1) / 2 * ((n_out + w - 1) / w), sms / 2) * (16 * 16 + w); };
     long cpair = m_blks >= 2 ? pair_cost(256) : (1L << 60);
-    if (c256 <= c128 && c256 <= cpair) return {SHAPE_256, 256};
-    if (c128 < cpair) return {SHAPE_128, 128};
+    if (c256 <= c128 && c256 <= cpair) return {SHAPE_256, 256, c256};
+    if (c128 < cpair) return {SHAPE_128, 128, c128};
     int bn = 256;
     for (int w = 256 - step; w >= 128; w -= step)
         if (pair_cost(w) < cpair) { cpair = pair_cost(w); bn = w; }
-    return {SHAPE_PAIR, bn};
+    return {SHAPE_PAIR, bn, cpair};
+}
+
+// Gate/up of a small canvas: as a stream of weights, or in the tiles above, which give the same bits.  The stream takes all tokens into
+// every SM with its share of the weights.  It is the faster one where the tiles take more than one wave of their smallest kind and the
+// stream takes in less than they do; tiles narrower than a pair's 256 columns are up to a twentieth better than their bytes.
+// Layers that are one wave of small tiles are not long enough for HBM to be what counts; there only the first rows are worth it.  A
+// step of four layers, tiles / stream, us (d_model x d_ff, rows): 4096 x 12288, 128: 632 / 627, 192: 734 / 712, 256: 794 / 823; 3584 x 18944,
+// 96: 632 / 630, 133: 717 / 680, 256: 807 / 799; 5120 x 13824, 112: 607 / 602, 256: 813 / 848; 2048 x 8192, 32: 241 / 238, 64: 242 / 250, 256: 331 / 377;
+// 2048 x 5632, 24: 232 / 228, 48: 228 / 238, 256: 304 / 364; 1024 x 4096, 32: 186 / 185, 48: 188 / 190, 256: 243 / 283; two layers of the tiny model,
+// 32: 76.0 / 74.5, 96: 83.4 / 86.4, 256: 104 / 116.
+bool stream_gateup_pays(int M, int n_out, int sms) {
+    if (M > kStreamMaxTokens) return false;
+    if (M <= 32) return true;
+    const ShapePick tiles = pick_shape(M, 2 * n_out, sms, 32);
+    const int rows = stream_gateup_rows(n_out, sms), units = (n_out + rows - 1) / rows;
+    const long cost = (long)((units + sms - 1) / sms) * (2 * rows + (M + 15) / 16 * 16) * 2;
+    const bool narrow = tiles.shape != SHAPE_PAIR || tiles.bn < 256;
+    return tiles.cost > 32 * 16 && (narrow ? cost * 20 <= tiles.cost * 19 : cost <= tiles.cost);
 }
 
 // Split-K factor for a plain projection: when 256-wide tiles leave most SMs idle, cut K into up to 4
@@ -525,7 +544,7 @@ struct jot_model {
     // A-operand maps of the projections for a pass over M rows (rows past M read as zero without memory
     // traffic): one set for the whole canvas, one for the rows of a block
     // (x*: the same buffers as the token operand of the slab kernel, boxes of half an accumulator's tokens)
-    struct ActMaps { int M = -1; bool slab = false, slab_gate_up = false, stream = false; CUtensorMap a, attn, act;
+    struct ActMaps { int M = -1; bool slab = false, slab_gate_up = false, stream = false, stream_gate_up = false; CUtensorMap a, attn, act;
                      SlabMaps xa, xattn, xact; CUtensorMap sa, sattn, sact; };
     ActMaps maps_full, maps_span;
     // block-wise KV cache (caller's memory, optional): per layer the rotated Q/K rows and V^T of the whole canvas
@@ -656,6 +675,7 @@ int encode_act_maps(jot_model* m, jot_model::ActMaps* am, int M) {
     JOT_TRY(make_map_2d(m->di, &am->act, m->act, M, c.d_ff, c.d_ff, 128));
     am->slab = M <= kSlabPreferTokens;
     am->stream = M <= kStreamMaxTokens;
+    am->stream_gate_up = stream_gateup_pays(M, c.d_ff, m->di->sms);
     am->slab_gate_up = (2 * c.d_ff) % 256 == 0 && slab2_plan(M, 2 * c.d_ff / 256, slab_cluster_capacity(m->di->sms, 1)).ok;
     if (am->stream) {
         const uint32_t tokens = (uint32_t)((M + 15) / 16 * 16);
@@ -770,7 +790,7 @@ int forward_body(jot_model* m, const int32_t* d_tokens, int B, int L, cudaStream
         {
             ProfScope ps(m, JOT_PROF_GEMM_GATE_UP, st);
             JOT_TRY(run_gemm(m->di, am.a, m->wgu[l], EPI_SWIGLU, p, st, nullptr, 0, nullptr,
-                             am.slab_gate_up ? &am.xa : nullptr, am.stream ? &am.sa : nullptr));
+                             am.slab_gate_up ? &am.xa : nullptr, am.stream_gate_up ? &am.sa : nullptr));
         }
         p = GemmParams{};
         p.M = M; p.N = d; p.K = c.d_ff; p.C = m->h; p.residual = m->h; p.ldc = d; p.status = status;
