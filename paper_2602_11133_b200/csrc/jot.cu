@@ -160,17 +160,28 @@ int launch_pair_t(const GemmParams& p, const CUtensorMap& tmA, const CUtensorMap
     return launch_check();
 }
 
-struct WeightMaps {     // one weight matrix as B operand, for both tile widths
-    CUtensorMap m128, m256;
-    const void* ptr;    // and what a map of another width is made from
+struct WeightMaps {     // one weight matrix as B operand
+    CUtensorMap m128, m256;     // for both tile widths
+    CUtensorMap stream;         // gate/up only: boxes of a stream's share of rows
+    CUtensorMap narrow;         // boxes of `narrow_rows` rows: the width that pair tiles had last, which hangs on the rows of the pass
+    int narrow_rows = 0;
+    const void* ptr;
     int rows, cols;
 };
 
 int make_weight_maps(const DeviceInfo* di, WeightMaps* w, const void* ptr, int rows, int cols, bool swiglu) {
-    w->ptr = ptr; w->rows = rows; w->cols = cols;
+    w->ptr = ptr; w->rows = rows; w->cols = cols; w->narrow_rows = 0;
     // swiglu tiles fetch gate and up rows as two boxes of half the tile width
     JOT_TRY(make_map_2d(di, &w->m128, ptr, rows, cols, cols, swiglu ? 64 : 128));
     JOT_TRY(make_map_2d(di, &w->m256, ptr, rows, cols, cols, swiglu ? 128 : 256));
+    if (swiglu) JOT_TRY(make_map_2d(di, &w->stream, ptr, rows, cols, cols, (uint32_t)stream_gateup_rows(rows / 2, di->sms)));
+    return JOT_OK;
+}
+int narrow_weight_map(const DeviceInfo* di, WeightMaps* w, int box_rows) {
+    if (w->narrow_rows == box_rows) return JOT_OK;
+    w->narrow_rows = 0;
+    JOT_TRY(make_map_2d(di, &w->narrow, w->ptr, w->rows, w->cols, w->cols, (uint32_t)box_rows));
+    w->narrow_rows = box_rows;
     return JOT_OK;
 }
 
@@ -264,10 +275,8 @@ int launch_stream(void (*kernel)(KArgs...), bool* attr_set, int ctas, int smem, 
 int run_stream_gateup(const DeviceInfo* di, const CUtensorMap& tmX, const WeightMaps& w, const GemmParams& p, cudaStream_t st) {
     static thread_local bool attr_set[64] = {};
     const int n_out = p.N / 2, rows = stream_gateup_rows(n_out, di->sms);
-    CUtensorMap tmW;
-    JOT_TRY(make_map_2d(di, &tmW, w.ptr, w.rows, w.cols, w.cols, (uint32_t)rows));
     return launch_stream(gemm_stream_gateup_kernel, attr_set, std::min(di->sms, (n_out + rows - 1) / rows),
-                         stream_geom(p.M, 2 * rows, (p.M + 15) / 16 * 16).smem_bytes, st, p, rows, tmW, tmX);
+                         stream_geom(p.M, 2 * rows, (p.M + 15) / 16 * 16).smem_bytes, st, p, rows, w.stream, tmX);
 }
 
 // How many clusters of `split` pairs the device runs side by side (1 CTA per SM: the kernel takes all shared memory).
@@ -427,7 +436,7 @@ int run_stream_partial(const CUtensorMap& tmX, const WeightMaps& w, GemmParams p
     return launch_reduce_norm(scratch, split, p, norm, 256, st);
 }
 
-int run_gemm(const DeviceInfo* di, const CUtensorMap& tmA, const WeightMaps& w, int epi, GemmParams p, cudaStream_t st,
+int run_gemm(const DeviceInfo* di, const CUtensorMap& tmA, WeightMaps& w, int epi, GemmParams p, cudaStream_t st,
              float* scratch = nullptr, size_t scratch_bytes = 0, NormAfter* norm = nullptr,
              const SlabMaps* tmX_slab = nullptr, const CUtensorMap* tmX_stream = nullptr) {
     int split_s = 0;
@@ -460,9 +469,8 @@ int run_gemm(const DeviceInfo* di, const CUtensorMap& tmA, const WeightMaps& w, 
         const long bands = 2ll * p.M * p.K <= kPairBandBytes ? 1 : (pair_rows + kPairBand - 1) / kPairBand;
         p.band = (int)((pair_rows + bands - 1) / bands);
         // each CTA of a pair fetches half of the tile's rows of W (SwiGLU: one its gate rows, the other its up rows)
-        CUtensorMap narrow;
-        if (pick.bn < 256) JOT_TRY(make_map_2d(di, &narrow, w.ptr, w.rows, w.cols, w.cols, (uint32_t)pick.bn / 2));
-        const CUtensorMap& tmB = pick.bn < 256 ? narrow : (epi == EPI_SWIGLU ? w.m256 : w.m128);
+        if (pick.bn < 256) JOT_TRY(narrow_weight_map(di, &w, pick.bn / 2));
+        const CUtensorMap& tmB = pick.bn < 256 ? w.narrow : (epi == EPI_SWIGLU ? w.m256 : w.m128);
         if (epi == EPI_STORE) return launch_pair_t<EPI_STORE>(p, tmA, tmB, grid, st);
         if (epi == EPI_QKV) return launch_pair_t<EPI_QKV>(p, tmA, tmB, grid, st);
         return launch_pair_t<EPI_SWIGLU>(p, tmA, tmB, grid, st);

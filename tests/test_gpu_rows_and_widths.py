@@ -117,6 +117,21 @@ def test_same_bits_of_both_norms(jot, d, heads, hd):
             assert torch.equal(x[0], y[b])
 
 
+# a model keeps what it knows of its weights between passes: passes of other rows in between (other widths of the pair tiles, streams,
+# slabs) change no bit
+def test_same_bits_whatever_came_before(jot):
+    g = geometry(512, 8, 64, 3968)
+    weights = inputs.model_weights(g, seed=0, device="cuda")
+    shapes = [(8, 200), (1, 200), (5, 130), (8, 200), (8, 125), (1, 40), (5, 130), (3, 200), (8, 125)]
+    model = jot.Model(g, weights, 8, 200)
+    for B, L in shapes:
+        tokens = masked_canvas(g, B, L, 8)
+        st = model.denoise_step(tokens, L - 8, L)
+        for got, want in zip((st.top1, st.top2, st.sumexp, st.argmax), statistics(jot, g, weights, tokens, L - 8)):
+            assert torch.equal(got[:, L - 8:], want)
+    model.close()
+
+
 # gate/up of fewer rows is less work and takes no longer: 257 to 352 rows of the LLaDA-8B widths against 384 (pair tiles of 224 columns
 # took 1.07 times as long), 96 to 256 rows of smaller layers against 300 (the stream of weights took up to 1.7 times as long)
 @pytest.mark.parametrize("d,heads,hd,ff,fewer,rows", [(4096, 32, 128, 12288, (257, 300, 352), 384), (2048, 16, 128, 5632, (64, 128, 256), 300),
