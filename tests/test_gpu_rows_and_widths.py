@@ -38,17 +38,24 @@ def geometry(d, heads, hd, ff, layers=2):
     return inputs.ModelGeometry(layers, d, heads, heads, hd, ff, 1032, 1000, 10000.0)
 
 
-# rows of the norm: one, two, three and more vectors per thread
-@pytest.mark.parametrize("d,B,L", [(64, 1, 20), (4096, 1, 20), (4160, 1, 20), (8256, 1, 20), (320, 9, 133)])     # ... and more rows than CTAs
+# rows of the norm: one, two, three and more vectors per thread; then more rows than CTAs with each of the three instances
+@pytest.mark.parametrize("d,B,L", [(64, 1, 20), (4096, 1, 20), (4160, 1, 20), (8256, 1, 20), (320, 9, 133), (4160, 3, 133), (8256, 2, 133)])
 def test_norm_widths(jot, d, B, L):
     check_step(jot, geometry(d, 2, 64, 128, layers=1), B, L)
 
 
 # pair tiles narrower than 256 columns: halves of 112 and of 64 gate columns, O and down in tiles of 240 and less; the last tile and
-# the last row block ragged; more row blocks than a band has
+# the last row block ragged
 @pytest.mark.parametrize("d,ff,B,L", [(256, 1984, 8, 125), (256, 1024, 8, 125), (512, 3968, 4, 130), (4096, 512, 8, 125), (256, 512, 18, 131)])
 def test_pair_tile_widths(jot, d, ff, B, L):
     check_step(jot, geometry(d, d // 64, 64, ff, layers=1), B, L)
+
+
+# activations that are walked in bands, an odd number of row blocks, the last band shorter: down (5 and 4 of 9 row-block pairs), then QKV
+# and gate/up (six times 8, then 2 of 50)
+@pytest.mark.parametrize("d,heads,ff,B,L", [(256, 4, 12032, 15, 140), (2048, 2, 640, 97, 130)])
+def test_bands(jot, d, heads, ff, B, L):
+    check_step(jot, geometry(d, heads, 64, ff, layers=1), B, L)
 
 
 # gate/up as two units per pair: a K of fewer blocks than stages, of as many, and more
@@ -59,17 +66,25 @@ def test_two_unit_gate_up(jot, d, B, L):
 
 
 # gate/up dealt over the SMs eight features at a time: 704 (a CTA of 8 each), 9600 (72, the last one ragged), 18944 (128 each), 19200 (two
-# units a CTA)
+# units a CTA); the larger passes of 704, 9600 and 19200 in tiles
 @pytest.mark.parametrize("ff", [704, 9600, 18944, 19200])
 @pytest.mark.parametrize("B,L", [(1, 1), (1, 16), (1, 17), (3, 11), (1, 128), (1, 144), (5, 29), (1, 255), (1, 256)])
 def test_small_canvases(jot, ff, B, L):
     check_step(jot, geometry(256, 4, 64, ff), B, L)
 
 
-# wide layers of few rows: four K ranges of O and down, a ragged last slab of 64 of 256 features
+# two and three units a CTA, both kinds of accumulators (two up to 128 rows); with 21 k-blocks the rings turn over inside a unit
+@pytest.mark.parametrize("d,ff", [(1344, 19200), (256, 38400), (1344, 38400)])
+@pytest.mark.parametrize("B,L", [(1, 17), (1, 128), (1, 144)])
+def test_several_units_a_cta(jot, d, ff, B, L):
+    check_step(jot, geometry(d, 4, 64, ff, layers=1), B, L)
+
+
+# wide layers of few rows, a ragged last slab of features: four, three and two K ranges of O and down
+@pytest.mark.parametrize("d", [1344, 4672, 6464])
 @pytest.mark.parametrize("B,L", [(1, 33), (1, 133), (2, 120)])
-def test_small_canvases_of_long_sums(jot, B, L):
-    check_step(jot, geometry(1344, 24, 128, 3200, layers=1), B, L)
+def test_small_canvases_of_long_sums(jot, d, B, L):
+    check_step(jot, geometry(d, 24, 128, 3200, layers=1), B, L)
 
 
 def statistics(jot, g, weights, tokens, lo):
