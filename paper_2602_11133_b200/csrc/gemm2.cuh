@@ -18,11 +18,14 @@ namespace jot {
 constexpr int kPairStages = 6;
 constexpr int kPairStageBytes = 2 * kBM * kBK * 2;                 // A tile + half W tile per CTA
 constexpr int kPairDynBytes = kPairStages * kPairStageBytes + 1024;
-// Tiles are walked in bands of at most this many row-block pairs where the activations are larger than kPairBandBytes: a band's rows
-// stay in L2 (126 MB, in two halves) while W streams past, where all rows in turn would come from HBM again for every column or two
-// of tiles.  11264 rows, one layer's projections at 12 / 8 / 6 / 4 / all 44 pairs a band: QKV 828 / 820 / 848 / 882 / 940 us, gate/up 1618 /
-// 1609 / 1652 / 1718 / 1821, down 851 / 847 / 870 / 904 / 960; the step 126.5 / 126.8 / 129.0 / 132.7 / 146.7 ms.  Activations that fit
-// would only read W once more per band: 4096 rows of 3584 (29 MB), gate/up 780 us in two bands, 768 in one.
+// Tiles are walked in bands of at most this many row-block pairs where the activations are larger than kPairBandBytes.  The 74 tiles that run
+// at once then are about 8 row-block pairs by 9 column blocks, and a k-block of all of them 17 tiles' worth of operands; all 44 pairs of 11264
+// rows by one or two columns are 46, and the activations come from HBM again for every column or two.  That does not hang on K, so the
+// band counts rows: with 78 MB a band (K = 18944) fewer rows are slower too.  A step at 4 / 6 / 8 / 12 / all row-block pairs a band, ms: LLaDA-8B
+// shape, 11264 rows 132.5 / 130.5 / 129.3 / 127.3 / 145.4, 8192 rows 94.6 / 92.9 / 91.7 / 91.2 / 97.1, 5632 rows (46 MB of activations but in down)
+// 63.9 / 63.7 / 63.9 / 63.9 / 64.2; Dream-7B shape, 11264 rows 120.1 / 118.5 / 118.1 / 117.2 / 128.9, of that down (K = 18944) 1170 / 1154 / 1137 / 1129 /
+// 1239 us a layer; 4096 rows 42.0 / 42.8 / 42.7 / 42.7 / 43.0.  Activations that fit L2 (126 MB, in two halves) would only read W once more per
+// band: 4096 rows of 3584 (29 MB), gate/up 780 us in two bands, 768 in one.
 constexpr int kPairBand = 8;
 constexpr long long kPairBandBytes = 48ll << 20;
 
@@ -87,7 +90,7 @@ gemm_pair_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmA, co
     grid_launch_dependents();
     if (is_stats(EPI)) grid_dependency_wait();
 
-    // ---- schedule: pair tiles (two row blocks x one 256-wide column block), identical in every role ----
+    // ---- schedule: pair tiles (two row blocks x one column block of bn), identical in every role ----
     const int num_m = (p.M + kBM - 1) / kBM, num_pm = (num_m + 1) / 2;
     const int bn_out = (EPI == EPI_SWIGLU) ? bn / 2 : bn;
     const int n_out = (EPI == EPI_SWIGLU) ? p.N / 2 : p.N;

@@ -33,10 +33,10 @@ namespace jot {
 
 constexpr int kSlabThreads = 320;
 constexpr int kSlabMaxTokens = 512;        // two accumulators of 256 fp32 columns fill tensor memory
-#ifndef JOT_SLAB_PREFER_TOKENS
-#define JOT_SLAB_PREFER_TOKENS 256
-#endif
-constexpr int kSlabPreferTokens = JOT_SLAB_PREFER_TOKENS;   // measured: up to here this kernel beats the token-major tiles
+// Up to here QKV and the last layer's down (and O and down where a stream's sums do not fit their scratch) run as slabs.  A step of four
+// layers with token-major tiles in their place, at 32 / 128 / 160 / 224 / 256 rows: LLaDA-8B shape +1.1 / -1.0 / +5.3 / +2.4 / -1.7 %, Dream-7B shape
+// +4.6 / +4.5 / +10.4 / +7.3 / +6.0, tiny model -0.6 / -3.1 / +3.8 / -1.7 / -3.4.
+constexpr int kSlabPreferTokens = 256;
 constexpr int kSlabMaxSmem = 226 * 1024;   // dynamic part; the static barriers take the rest of the 227 KB
 enum { SLAB_STORE = 0, SLAB_SWIGLU = 1, SLAB_QKV = 2 };      // (SLAB_SWIGLU: the two-unit kernel below)
 
@@ -100,7 +100,7 @@ gemm_slab_kernel(const GemmParams p, const __grid_constant__ CUtensorMap tmW, co
     const int pr = (int)(rank & 1u), ks = (int)(rank >> 1);     // rank inside the pair, K range of the pair
     const uint32_t leader_rank = rank & ~1u;
     const bool leader = pr == 0;
-    const int slab = p.slab0 + (int)(blockIdx.x / (2 * split)); // pair-slab: 256 weight rows (128 outputs for SwiGLU)
+    const int slab = p.slab0 + (int)(blockIdx.x / (2 * split)); // pair-slab: 256 weight rows
     const SlabGeom g = slab_geom(p.M, split);
     const int stages = g.stages;
     const int h0 = g.n0 / 2, h1 = g.n1 / 2;                      // token rows this CTA loads per accumulator
