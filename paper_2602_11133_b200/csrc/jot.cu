@@ -418,30 +418,36 @@ int launch_reduce_norm(const float* scratch, int split, const GemmParams& p, Nor
 }
 
 // A projection with residual whose output is normalised next, as a stream of weights in K ranges over the CTA pairs.  Needs
-// `scratch` for the ranges' sums.  The ranges are the slab kernel's and the norm's threads are rmsnorm_kernel's, which take these rows
-// where the sums do not fit `scratch`: both routes add in the same order and give the same bits.  (Ranges for as many pairs as there
-// are SMs, and a thread per vector in the norm: 5 rows of the LLaDA-8B shape 2 % faster, other steps of up to 256 rows of three
-// shapes 1.4 % faster to 0.9 % slower.)
-bool stream_split(const DeviceInfo* di, const GemmParams& p, size_t scratch_bytes, const NormAfter* norm, int* split) {
+// `scratch` for the ranges' sums.  Up to 128 rows the ranges are the slab kernel's, which takes these rows where the sums do not fit, and
+// whenever they are the norm's threads are rmsnorm_kernel's (256): both routes add in the same order and give the same bits.  Beyond, as
+// many ranges as there are pairs for, and a thread per vector in the norm where that makes it another order anyhow: 133 / 256 rows of the
+// LLaDA-8B shape (four ranges for three), eight layers, 1161 / 1476 -> 1145 / 1460 us.
+bool stream_split(const DeviceInfo* di, const GemmParams& p, size_t scratch_bytes, const NormAfter* norm, int* split, int* norm_threads) {
     if (!norm || p.ldc != p.N || p.N / 8 > 1024 || p.M > kStreamMaxTokens) return false;
-    *split = slab_pick_split(p.M, (p.N + 255) / 256, (p.K + kBK - 1) / kBK, di->sms);
+    const int slabs = (p.N + 255) / 256, num_kb = (p.K + kBK - 1) / kBK;
+    const int slab_split = slab_pick_split(p.M, slabs, num_kb, di->sms);
+    *split = slab_split;
+    if (p.M > 128)
+        for (*split = std::min(4, di->sms / 2 / slabs); *split > 1 && num_kb / *split < 8;) --*split;
+    *norm_threads = *split == slab_split ? 256 : 512;
     return (size_t)*split * p.M * p.N * 4 <= scratch_bytes;
 }
-int run_stream_partial(const CUtensorMap& tmX, const WeightMaps& w, GemmParams p, int split, float* scratch, NormAfter* norm, cudaStream_t st) {
+int run_stream_partial(const CUtensorMap& tmX, const WeightMaps& w, GemmParams p, int split, int norm_threads, float* scratch, NormAfter* norm,
+                       cudaStream_t st) {
     static thread_local bool attr_set[64] = {};
     p.split_k = split;
     p.partial = scratch;
     JOT_TRY(launch_stream(gemm_stream_partial_kernel, attr_set, 2 * split * ((p.N + 255) / 256), stream_geom(p.M, 128, (p.M + 15) / 16 * 8).smem_bytes, st,
                           p, w.m128, tmX));
-    return launch_reduce_norm(scratch, split, p, norm, 256, st);
+    return launch_reduce_norm(scratch, split, p, norm, norm_threads, st);
 }
 
 int run_gemm(const DeviceInfo* di, const CUtensorMap& tmA, WeightMaps& w, int epi, GemmParams p, cudaStream_t st,
              float* scratch = nullptr, size_t scratch_bytes = 0, NormAfter* norm = nullptr,
              const SlabMaps* tmX_slab = nullptr, const CUtensorMap* tmX_stream = nullptr) {
-    int split_s = 0;
-    if (tmX_stream && epi == EPI_STORE && stream_split(di, p, scratch_bytes, norm, &split_s))
-        return run_stream_partial(*tmX_stream, w, p, split_s, scratch, norm, st);
+    int split_s = 0, norm_threads = 0;
+    if (tmX_stream && epi == EPI_STORE && stream_split(di, p, scratch_bytes, norm, &split_s, &norm_threads))
+        return run_stream_partial(*tmX_stream, w, p, split_s, norm_threads, scratch, norm, st);
     if (tmX_stream && epi == EPI_SWIGLU) return run_stream_gateup(di, *tmX_stream, w, p, st);
     // small canvases: weight rows as the MMA's M side, every token in tensor memory (gemm_slab.cuh)
     if (tmX_slab && p.M <= kSlabMaxTokens) return run_slab(di, *tmX_slab, w, epi, p, st);      // callers decide when

@@ -101,9 +101,9 @@ def masked_canvas(g, B, L, n_masked):
 
 
 # down adds the same K ranges in the same order with a norm behind it (streams) and as the last layer's (slabs): a second layer that
-# adds nothing changes no bit
-@pytest.mark.parametrize("d,heads,hd,ff", [(256, 4, 64, 704), (3584, 28, 128, 2048), (4096, 32, 128, 3072), (4672, 4, 64, 2048), (8192, 4, 64, 1088)])
-@pytest.mark.parametrize("L", [20, 133, 256])
+# adds nothing changes no bit.  (4096 columns have a range more beyond 128 rows.)
+@pytest.mark.parametrize("d,heads,hd,ff,L", [(4096, 32, 128, 3072, L) for L in (20, 96, 128)] + [
+    (*widths, L) for widths in ((256, 4, 64, 704), (3584, 28, 128, 2048), (4672, 4, 64, 2048), (8192, 4, 64, 1088)) for L in (20, 128, 133, 256)])
 def test_same_bits_with_a_norm_behind_and_without(jot, d, heads, hd, ff, L):
     g = geometry(d, heads, hd, ff)
     weights = inputs.model_weights(g, seed=0, device="cuda")
