@@ -118,17 +118,19 @@ def test_same_bits_with_a_norm_behind_and_without(jot, d, heads, hd, ff, L):
 
 # the norm in the tail of a split projection adds a row's squares in the order of the norm on its own: a sequence gets the same bits
 # alone and in a batch, where no projection is split (O and down have one K range that is not zero, so that their sums are the same)
+# (20 rows have gate/up as a stream, the others in tiles.)
 @pytest.mark.parametrize("d,heads,hd", [(3584, 28, 128), (4096, 32, 128), (5120, 32, 128)])
-def test_same_bits_of_both_norms(jot, d, heads, hd):
+@pytest.mark.parametrize("B,L", [(9, 100), (45, 20)])
+def test_same_bits_of_both_norms(jot, d, heads, hd, B, L):
     g = geometry(d, heads, hd, 4096)
     weights = inputs.model_weights(g, seed=0, device="cuda")
     for layer in weights["layers"]:
         layer["wo"][:, heads * hd // 256 * 64:] = 0
         layer["w_down"][:, g.d_ff // 4:] = 0
-    tokens = masked_canvas(g, 9, 100, 8)
-    batch = statistics(jot, g, weights, tokens, 92)
-    for b in (0, 8):
-        for x, y in zip(statistics(jot, g, weights, tokens[b:b + 1].contiguous(), 92), batch):
+    tokens = masked_canvas(g, B, L, 2)
+    batch = statistics(jot, g, weights, tokens, L - 2)
+    for b in (0, B - 1):
+        for x, y in zip(statistics(jot, g, weights, tokens[b:b + 1].contiguous(), L - 2), batch):
             assert torch.equal(x[0], y[b])
 
 
